@@ -376,35 +376,82 @@ void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, int64_t rows
                                                        o.rows_valid);
 }
 
+// ---------------------------------------------------------------------------
+// Stand-alone measurement: a block of four warps takes R rows.  First the w_s of its rows, one thread per
+// (row, outcome); then one thread per row draws; then all threads write the rows; the logarithm comes last.
+// Bound by HBM: one selected block read and one next row written per sample.  131072 rows of 512 entries
+// (d = 4, BF16 planes): 94 us = 5.8 TB/s; 65536 rows of 2048 entries: 180 us = 6.0 TB/s in BF16 planes,
+// 201 us in FP16.  (One warp for 32 rows in turn, its draw included: 110, -- and 516 us; and 398 us against
+// 24 where a call has 5003 rows of 1554 entries, because 157 warps were all there was.)
+// ---------------------------------------------------------------------------
 constexpr int MEASURE_THREADS = 128;
-constexpr int MEASURE_WARPS = MEASURE_THREADS / 32;
+constexpr int MEASURE_ROWS = 32;    // most rows of a block
+constexpr int MEASURE_SUMS = 1024;  // most (row, outcome) sums of a block
 
-// Stand-alone measurement (FP32 path, and BF16 paths when not fused): a warp
-// handles 32 samples, one per lane for the draw, then the warp writes each
-// sample's next left row with coalesced loads.
-__global__ void __launch_bounds__(MEASURE_THREADS) measure_kernel(const MeasureArgs a) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int base = (blockIdx.x * MEASURE_WARPS + warp) * 32;
-    if (base >= a.rows) return;
-    const int row = base + lane;
-    int sstar = 0;
-    float scale = 0.f;
-    if (row < a.rows) sstar = measure_draw(a, row, &scale);
-    const int count = min(32, a.rows - base);
-    for (int j = 0; j < count; ++j) {
-        const int sj = __shfl_sync(0xffffffffu, sstar, j);
-        const float scj = __shfl_sync(0xffffffffu, scale, j);
-        const int r = base + j;
-        const float *ysrc = a.Y + (int64_t)r * a.ldY + (int64_t)sj * a.Cs;
-        measure_write_row(a, lane, ysrc, scj, a.row0 + r);
+// kScaled: FP16 or E4M3 rows (one warp per row), else FP32 or BF16 planes
+template <bool kScaled>
+__global__ void __launch_bounds__(MEASURE_THREADS) measure_kernel(const MeasureArgs a, int R) {
+    __shared__ double w_sh[MEASURE_SUMS];
+    __shared__ int sstar_sh[MEASURE_ROWS];
+    __shared__ float scale_sh[MEASURE_ROWS];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int r0 = blockIdx.x * R;
+    const int count = min(R, a.rows - r0);
+    const int T = a.tiles_per_s, d = a.d;
+    for (int q = tid; q < count * d; q += MEASURE_THREADS) {
+        const int r = q / d, s = q - r * d;
+        w_sh[q] = sum_tiles(a.P + (int64_t)(r0 + r) * a.ldP + s * T, T);
     }
+    double u = 0.0, lp = 0.0;
+    if (tid < count) {
+        u = sample_uniform(a.seed, a.n_base + (uint64_t)(r0 + tid), a.k, a.job);
+        lp = a.logp[a.row0 + r0 + tid];
+    }
+    __syncthreads();
+    double Z = 0.0, ws = 0.0;
+    bool ok = false;
+    if (tid < count) {
+        const double *w = w_sh + tid * d;
+        for (int s = 0; s < d; ++s) Z += w[s];
+        const double t = u * Z;
+        double C = 0.0;
+        int sstar = d - 1;
+        for (int s = 0; s < d; ++s) {
+            C += w[s];
+            if (s == d - 1 || C >= t) {
+                sstar = s;
+                ws = w[s];
+                break;
+            }
+        }
+        ok = (Z > 0.0) && isfinite(Z) && (ws > 0.0);
+        sstar_sh[tid] = sstar;
+        scale_sh[tid] = ok ? rsqrtf((float)ws) : 0.f;
+        a.outcomes[r0 + tid] = (uint8_t)sstar;
+    }
+    __syncthreads();
+    if constexpr (!kScaled) {
+        write_rows_flat(a, tid, MEASURE_THREADS, r0, count, sstar_sh, scale_sh);
+    } else {
+        for (int j = tid >> 5; j < count; j += MEASURE_THREADS / 32)
+            write_row_scaled(a, lane, a.Y + (int64_t)(r0 + j) * a.ldY + (int64_t)sstar_sh[j] * a.Cs, scale_sh[j],
+                             a.row0 + r0 + j);
+    }
+    // nothing waits for the logarithm: it follows the row writes
+    if (tid < count) measure_finish(a, r0 + tid, ws, Z, ok, lp, w_sh + tid * d);
 }
 
 void launch_measure(const MeasureArgs &a, cudaStream_t st) {
     if (a.rows <= 0) return;
-    const int rows_per_block = MEASURE_WARPS * 32;
-    const int grid = (a.rows + rows_per_block - 1) / rows_per_block;
-    measure_kernel<<<grid, MEASURE_THREADS, 0, st>>>(a);
+    // Rows per block: a warp's worth, so that the FP64 draw (a warp-wide FP64 instruction costs the SM 16
+    // cycles however many lanes it has) stays a small part; fewer where rows are wide (65536 rows of 2048
+    // entries: 204 us with 32 rows per block, 180 with 16) or where that would leave less than four blocks
+    // per SM (5003 rows of 1554 entries: 60 us with 32, 24 with 8); at most MEASURE_SUMS sums.
+    int R = MEASURE_ROWS;
+    while (R > 4 && (R * a.K_next > 32768 || (a.rows + R - 1) / R < 4 * 152 || R * a.d > MEASURE_SUMS)) R >>= 1;
+    const int grid = (a.rows + R - 1) / R;
+    if (a.f16 || a.V8) measure_kernel<true><<<grid, MEASURE_THREADS, 0, st>>>(a, R);
+    else measure_kernel<false><<<grid, MEASURE_THREADS, 0, st>>>(a, R);
 }
 
 // ---------------------------------------------------------------------------

@@ -24,10 +24,11 @@ namespace fastmps {
 //    are taken in FP64 (one log per sample per site, O(N M) work), since a
 //    rare outcome has w_{s*} << 1 and the absolute error of an FP32 log
 //    there would add up over thousands of sites.
-// Phase 2, a warp per sample (measure_write_row): the selected block y_{s*} is scaled
-// by 1/sqrt(w_{s*}) (FP32; the scale cancels in every later ratio w/Z) and
-// written as the next left row -- FP32, or BF16 planes of successive
-// residuals -- with coalesced 16-byte loads.
+// Phase 2, a group of warps for a group of rows (measure_write_rows): the selected block y_{s*} of
+// each row is scaled by 1/sqrt(w_{s*}) (FP32; the scale cancels in every later ratio w/Z) and
+// written as the next left row -- FP32, or BF16 planes of successive residuals -- with coalesced
+// 32-byte loads.  FP16 and E4M3 rows, whose power-of-two scale comes from the row's largest entry, are
+// read twice by one warp.
 // GB300's FP64 pipes are narrow, so FP64 is kept to the O(d) per-sample
 // operations of the draw and the accumulation, one sample per lane.
 // ---------------------------------------------------------------------------
@@ -40,111 +41,190 @@ __device__ __forceinline__ void write_planes(float x, int nplanes, __nv_bfloat16
     if (nplanes < 3) h2 = __float2bfloat16_rn(0.f);
 }
 
-__device__ __forceinline__ void measure_write_row(const MeasureArgs &a, int lane, const float *ysrc, float scale,
-                                                  int64_t grow) {
-    const int nreal = 2 * a.chi_r;
+// Eight entries (columns i .. i+7, i a multiple of 8) of a selected block; zero at and beyond nreal.
+// One 32-byte load through L2 (the block may have been written by other thread blocks of the same
+// kernel).  A block's columns are padded to a multiple of 32 (SiteLayout::Cs), so the load at i < nreal
+// stays inside the block, and is 32-byte aligned, for any nreal.
+struct Entries8 {
+    float x[8];
+};
+
+__device__ __forceinline__ Entries8 load_block8(const float *ysrc, int i, int nreal) {
+    Entries8 v;
+    if (i >= nreal) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v.x[e] = 0.f;
+        return v;
+    }
+    asm volatile("ld.global.cg.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v.x[0]), "=f"(v.x[1]), "=f"(v.x[2]), "=f"(v.x[3]), "=f"(v.x[4]), "=f"(v.x[5]), "=f"(v.x[6]),
+                   "=f"(v.x[7])
+                 : "l"(ysrc + i)
+                 : "memory");
+    if (i + 7 >= nreal) {
+#pragma unroll
+        for (int e = 1; e < 8; ++e)
+            if (i + e >= nreal) v.x[e] = 0.f;
+    }
+    return v;
+}
+
+// Entries i .. i+7 of a next left row in FP32 or BF16 planes (off: element offset of entry i).
+__device__ __forceinline__ void store_row8(const MeasureArgs &a, int64_t off, const Entries8 &v, float scale) {
     if (a.V32) {
-        float *dst = a.V32 + grow * a.ld_next;
-        if ((nreal & 3) == 0) {
-            constexpr int U = 4;
-            for (int base = 4 * lane; base < a.K_next; base += 128 * U) {
-                float4 v[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int i = base + 128 * u;
-                    v[u] = i < nreal ? __ldcg(reinterpret_cast<const float4 *>(ysrc + i))
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int i = base + 128 * u;
-                    if (i >= a.K_next) break;
-                    *reinterpret_cast<float4 *>(dst + i) =
-                        make_float4(v[u].x * scale, v[u].y * scale, v[u].z * scale, v[u].w * scale);
-                }
-            }
-        } else {
-            for (int i = lane; i < a.K_next; i += 32) dst[i] = i < nreal ? ysrc[i] * scale : 0.f;
-        }
+        float4 *dst = reinterpret_cast<float4 *>(a.V32 + off);
+        dst[0] = make_float4(v.x[0] * scale, v.x[1] * scale, v.x[2] * scale, v.x[3] * scale);
+        dst[1] = make_float4(v.x[4] * scale, v.x[5] * scale, v.x[6] * scale, v.x[7] * scale);
         return;
     }
+    __align__(16) __nv_bfloat16 p0[8], p1[8], p2[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) write_planes(v.x[e] * scale, a.nplanes, p0[e], p1[e], p2[e]);
+    *reinterpret_cast<uint4 *>(a.Vp[0] + off) = *reinterpret_cast<const uint4 *>(p0);
+    *reinterpret_cast<uint4 *>(a.Vp[1] + off) = *reinterpret_cast<const uint4 *>(p1);
+    if (a.nplanes > 2) *reinterpret_cast<uint4 *>(a.Vp[2] + off) = *reinterpret_cast<const uint4 *>(p2);
+}
+
+// Next left rows of micro-batch rows r0 .. r0+count-1 (FP32 or BF16 planes) by `nt` threads: the rows'
+// 8-entry pieces are dealt to the threads in order, so threads stay busy whether rows are 64 or 4096
+// entries wide.  sstar, scale: per row.  Pieces of 8 entries make every load 32 bytes and every BF16
+// plane store 16 bytes; more in flight per thread costs registers, so resident warps, and gains nothing.
+// 131072 rows of 512 entries (measurement kernel, 32 rows per block): 94 us with one 8-entry piece at a
+// time, 98 us with two, 137 us with four of 4 entries (16-byte loads, 8-byte stores).
+__device__ __forceinline__ void write_rows_flat(const MeasureArgs &a, int tid, int nt, int r0, int count,
+                                                const int *sstar, const float *scale) {
+    const int nreal = 2 * a.chi_r;
+    const int per_row = a.K_next >> 3;
+    const int step_r = nt / per_row, step_c = nt - step_r * per_row;
+    int r = tid / per_row, c = tid - r * per_row;
+    while (r < count) {
+        const Entries8 v = load_block8(a.Y + (int64_t)(r0 + r) * a.ldY + (int64_t)sstar[r] * a.Cs, 8 * c, nreal);
+        store_row8(a, (a.row0 + r0 + r) * (int64_t)a.ld_next + 8 * c, v, scale[r]);
+        r += step_r;
+        c += step_c;
+        if (c >= per_row) {
+            c -= per_row;
+            ++r;
+        }
+    }
+}
+
+// One FP16 or E4M3 next left row by one warp, read twice (for its largest entry, then for the entries;
+// the second read hits L2) in pieces of 512 entries; a row of one piece stays in registers.  Holding up to
+// 2048 entries in registers instead takes 229 us, not 201, for 65536 rows of 2048 entries: fewer warps are
+// resident.  The unit-norm row is scaled by the power of two that puts its largest entry in [top/2, top] -- top = 32768 for binary16, 448 for E4M3 -- which cancels
+// in w/Z at the next site and keeps small entries normal; then
+//   FP16: two binary16 planes of successive residuals, each rounded to nearest even;
+//   E4M3: one plane, or two with the residual at the same scale (the products add up to (V0 + V1) B).
+__device__ __forceinline__ void store_scaled8(const MeasureArgs &a, int64_t off, const Entries8 &v, float s2) {
     if (a.f16) {
-        // FP16 row: scale the unit-norm row by the power of two that puts its largest entry in
-        // [16384, 32768] (the scale cancels in w/Z at the next site; small entries stay normal), then
-        // two binary16 planes of successive residuals, each rounded to nearest even
-        float m = 0.f;
-        for (int i = lane; i < nreal; i += 32) m = fmaxf(m, fabsf(__ldcg(ysrc + i) * scale));
+        __align__(16) uint16_t h0[8], h1[8];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        const float s16 = m > 0.f ? exp2f(floorf(log2f(32768.f / m))) : 1.f;
-        uint16_t *d0 = reinterpret_cast<uint16_t *>(a.Vp[0]) + grow * a.ld_next;
-        uint16_t *d1 = reinterpret_cast<uint16_t *>(a.Vp[1]) + grow * a.ld_next;
-        for (int i = lane; i < a.K_next; i += 32) {
-            const float x = i < nreal ? (__ldcg(ysrc + i) * scale) * s16 : 0.f;
+        for (int e = 0; e < 8; ++e) {
+            const float x = v.x[e] * s2;
             const __half h = __float2half_rn(x);
-            d0[i] = __half_as_ushort(h);
-            d1[i] = __half_as_ushort(__float2half_rn(x - __half2float(h)));
+            h0[e] = __half_as_ushort(h);
+            h1[e] = __half_as_ushort(__float2half_rn(x - __half2float(h)));
         }
+        *reinterpret_cast<uint4 *>(a.Vp[0] + off) = *reinterpret_cast<const uint4 *>(h0);
+        *reinterpret_cast<uint4 *>(a.Vp[1] + off) = *reinterpret_cast<const uint4 *>(h1);
         return;
     }
-    if (a.V8) {
-        // E4M3 row: scale the unit-norm row by the power of two that puts its largest entry in
-        // [224, 448] (the scale cancels in w/Z at the next site), then round to nearest even
-        float m = 0.f;
-        for (int i = lane; i < nreal; i += 32) m = fmaxf(m, fabsf(__ldcg(ysrc + i) * scale));
+    __align__(8) uint8_t q0[8], q1[8];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        const float s8 = m > 0.f ? exp2f(floorf(log2f(448.f / m))) : 1.f;
-        uint8_t *dst = a.V8 + grow * a.ld_next;
-        uint8_t *dlo = a.V8lo ? a.V8lo + grow * a.ld_next : nullptr;
-        for (int i = lane; i < a.K_next; i += 32) {
-            const float x = i < nreal ? __ldcg(ysrc + i) * scale * s8 : 0.f;
-            const __nv_fp8_storage_t h = __nv_cvt_float_to_fp8(x, __NV_SATFINITE, __NV_E4M3);
-            dst[i] = (uint8_t)h;
-            if (dlo) {
-                // residual at the same scale: the two planes' products add up to (V0 + V1) B
-                const float hv = __half2float(__half(__nv_cvt_fp8_to_halfraw(h, __NV_E4M3)));
-                dlo[i] = (uint8_t)__nv_cvt_float_to_fp8(x - hv, __NV_SATFINITE, __NV_E4M3);
-            }
-        }
-        return;
+    for (int e = 0; e < 8; ++e) {
+        const float x = v.x[e] * s2;
+        const __nv_fp8_storage_t h = __nv_cvt_float_to_fp8(x, __NV_SATFINITE, __NV_E4M3);
+        q0[e] = (uint8_t)h;
+        const float hv = __half2float(__half(__nv_cvt_fp8_to_halfraw(h, __NV_E4M3)));
+        q1[e] = (uint8_t)__nv_cvt_float_to_fp8(x - hv, __NV_SATFINITE, __NV_E4M3);
     }
-    __nv_bfloat16 *d0 = a.Vp[0] + grow * a.ld_next;
-    __nv_bfloat16 *d1 = a.Vp[1] + grow * a.ld_next;
-    __nv_bfloat16 *d2 = a.nplanes > 2 ? a.Vp[2] + grow * a.ld_next : nullptr;
-    if ((nreal & 3) == 0) {
-        // four 16-byte loads in flight per lane before any store
-        constexpr int U = 4;
-        for (int base = 4 * lane; base < a.K_next; base += 128 * U) {
-            float4 v[U];
+    *reinterpret_cast<uint2 *>(a.V8 + off) = *reinterpret_cast<const uint2 *>(q0);
+    if (a.V8lo) *reinterpret_cast<uint2 *>(a.V8lo + off) = *reinterpret_cast<const uint2 *>(q1);
+}
+
+__device__ __forceinline__ void write_row_scaled(const MeasureArgs &a, int lane, const float *ysrc, float scale,
+                                                 int64_t grow) {
+    constexpr int NV = 2;  // 8-entry pieces per lane
+    const int nreal = 2 * a.chi_r;
+    const int64_t off = grow * a.ld_next;
+    Entries8 v[NV];
+    float m = 0.f;
+    auto take = [&](int base) {
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int i = base + 128 * u;
-                v[u] = i < nreal ? __ldcg(reinterpret_cast<const float4 *>(ysrc + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+        for (int u = 0; u < NV; ++u) v[u] = load_block8(ysrc, base + 8 * lane + 256 * u, nreal);
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int i = base + 128 * u;
-                if (i >= a.K_next) break;
-                const float x[4] = {v[u].x * scale, v[u].y * scale, v[u].z * scale, v[u].w * scale};
-                __align__(8) __nv_bfloat16 p0[4], p1[4], p2[4];
+        for (int u = 0; u < NV; ++u)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) write_planes(x[e], a.nplanes, p0[e], p1[e], p2[e]);
-                *reinterpret_cast<uint2 *>(d0 + i) = *reinterpret_cast<const uint2 *>(p0);
-                *reinterpret_cast<uint2 *>(d1 + i) = *reinterpret_cast<const uint2 *>(p1);
-                if (d2) *reinterpret_cast<uint2 *>(d2 + i) = *reinterpret_cast<const uint2 *>(p2);
-            }
+            for (int e = 0; e < 8; ++e) v[u].x[e] *= scale;
+    };
+    auto put = [&](int base, float s2) {
+#pragma unroll
+        for (int u = 0; u < NV; ++u) {
+            const int i = base + 8 * lane + 256 * u;
+            if (i >= a.K_next) break;
+            store_scaled8(a, off + i, v[u], s2);
         }
+    };
+    const bool one_piece = a.K_next <= 256 * NV;
+    for (int base = 0; base < nreal; base += 256 * NV) {
+        take(base);
+#pragma unroll
+        for (int u = 0; u < NV; ++u)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) m = fmaxf(m, fabsf(v[u].x[e]));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const float s2 = m > 0.f ? exp2f(floorf(log2f((a.f16 ? 32768.f : 448.f) / m))) : 1.f;
+    if (one_piece) {
+        put(0, s2);
     } else {
-        for (int i = lane; i < a.K_next; i += 32) {
-            const float x = i < nreal ? ysrc[i] * scale : 0.f;
-            __nv_bfloat16 h0, h1, h2;
-            write_planes(x, a.nplanes, h0, h1, h2);
-            d0[i] = h0;
-            d1[i] = h1;
-            if (d2) d2[i] = h2;
+        for (int base = 0; base < a.K_next; base += 256 * NV) {
+            take(base);
+            put(base, s2);
         }
     }
+}
+
+// Next left rows of micro-batch rows r0 .. r0+count-1 by `nt` threads (whole warps), any precision.
+__device__ __forceinline__ void measure_write_rows(const MeasureArgs &a, int tid, int nt, int r0, int count,
+                                                   const int *sstar, const float *scale) {
+    if (a.f16 || a.V8) {
+        for (int j = tid >> 5; j < count; j += nt >> 5)
+            write_row_scaled(a, tid & 31, a.Y + (int64_t)(r0 + j) * a.ldY + (int64_t)sstar[j] * a.Cs, scale[j],
+                                a.row0 + r0 + j);
+        return;
+    }
+    write_rows_flat(a, tid, nt, r0, count, sstar, scale);
+}
+
+// w_s of one row: the FP64 sum, in tile order, of its T per-tile sums of squares.  P is read through L2
+// (it may have been written by other thread blocks of the same kernel); eight loads are in flight.
+__device__ __forceinline__ double sum_tiles(const float *P, int T) {
+    double acc = 0.0;
+    int j = 0;
+    for (; j + 8 <= T; j += 8) {
+        float x[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = __ldcg(P + j + e);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc += (double)x[e];
+    }
+    for (; j < T; ++j) acc += (double)__ldcg(P + j);
+    return acc;
+}
+
+// Log-probability, numeric check and optional trace of one drawn row (w: its d sums, Z their total).
+__device__ __forceinline__ void measure_finish(const MeasureArgs &a, int row, double ws, double Z, bool ok, double lp,
+                                               const double *w) {
+    const int64_t grow = a.row0 + row;
+    if (ok) a.logp[grow] = lp + log(ws / Z);
+    else atomicExch(a.err, (int)kDevNumeric);
+    const int64_t slot = a.trace ? (a.trace_slot ? (int64_t)a.trace_slot[grow] : (grow < a.trace_rows ? grow : -1))
+                                 : -1;
+    if (slot >= 0)
+        for (int s = 0; s < a.d; ++s) a.trace[slot * a.d + s] = ok ? w[s] / Z : 0.0;
 }
 
 // Phase 1 for sample `row` of the micro-batch (row < a.rows): draw, outcome,
@@ -159,11 +239,7 @@ __device__ __forceinline__ int measure_draw(const MeasureArgs &a, int row, float
         const int T = a.tiles_per_s;
         // pass 1: Z = w_0 + ... + w_{d-1} in s order
         double Z = 0.0;
-        for (int s = 0; s < a.d; ++s) {
-            double acc = 0.0;
-            for (int j = 0; j < T; ++j) acc += (double)__ldcg(Prow + s * T + j);
-            Z += acc;
-        }
+        for (int s = 0; s < a.d; ++s) Z += sum_tiles(Prow + s * T, T);
         const uint64_t n = a.n_base + (uint64_t)row;
         const double t = sample_uniform(a.seed, n, a.k, a.job) * Z;
         // pass 2: the same partial sums again; s* is the first s < d-1 with C_s >= t (else d-1),
@@ -171,8 +247,7 @@ __device__ __forceinline__ int measure_draw(const MeasureArgs &a, int row, float
         double C = 0.0, ws = 0.0;
         sstar = a.d - 1;
         for (int s = 0; s < a.d; ++s) {
-            double acc = 0.0;
-            for (int j = 0; j < T; ++j) acc += (double)__ldcg(Prow + s * T + j);
+            const double acc = sum_tiles(Prow + s * T, T);
             C += acc;
             if (s == a.d - 1 || C >= t) {
                 sstar = s;
@@ -189,8 +264,7 @@ __device__ __forceinline__ int measure_draw(const MeasureArgs &a, int row, float
                                      : -1;
         if (slot >= 0) {
             for (int s = 0; s < a.d; ++s) {
-                double acc = 0.0;
-                for (int j = 0; j < T; ++j) acc += (double)__ldcg(Prow + s * T + j);
+                const double acc = sum_tiles(Prow + s * T, T);
                 a.trace[slot * a.d + s] = ok ? acc / Z : 0.0;
             }
         }

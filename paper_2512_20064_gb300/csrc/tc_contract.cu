@@ -870,7 +870,6 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
     } else if (kFused) {
         // ---------------- measurement: warps 6..9 ----------------
         const int m = threadIdx.x - 192;  // 0..127: the row of the m-tile this thread draws
-        const int mw = m >> 5;
         int ring = 0;
         uint32_t ring_phase = 0;
         while (true) {
@@ -893,13 +892,7 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
             m_sstar[m] = sstar;
             m_scale[m] = scale;
             named_bar_sync(2, 128);
-            for (int j = 0; j < 32; ++j) {
-                const int r = mt * kBM + mw * 32 + j;
-                if (r >= p.rows_valid) break;
-                const int sj = m_sstar[mw * 32 + j];
-                const float *ysrc = p.Y + (int64_t)r * p.ldY + (int64_t)sj * p.m.Cs;
-                measure_write_row(p.m, lane, ysrc, m_scale[mw * 32 + j], p.m.row0 + r);
-            }
+            measure_write_rows(p.m, m, 128, mt * kBM, min(kBM, p.rows_valid - mt * kBM), m_sstar, m_scale);
             named_bar_sync(2, 128);
         }
     }

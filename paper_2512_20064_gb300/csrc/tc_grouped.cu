@@ -393,7 +393,6 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
     } else {
         // ---------------- measurement: warps 6..9 ----------------
         const int m = threadIdx.x - 192;  // the row of the m-tile this thread draws
-        const int mw = m >> 5;
         int ring = 0;
         uint32_t ring_phase = 0;
         while (true) {
@@ -419,13 +418,7 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
             m_sstar[m] = sstar;
             m_scale[m] = scale;
             named_bar_sync(2, 128);
-            for (int j = 0; j < 32; ++j) {
-                const int r = mt * kBM + mw * 32 + j;
-                if (r >= rows) break;
-                const int sj = m_sstar[mw * 32 + j];
-                const float *ysrc = a.Y + (int64_t)r * a.ldY + (int64_t)sj * a.Cs;
-                measure_write_row(a, lane, ysrc, m_scale[mw * 32 + j], a.row0 + r);
-            }
+            measure_write_rows(a, m, 128, mt * kBM, min(kBM, rows - mt * kBM), m_sstar, m_scale);
             named_bar_sync(2, 128);  // the m-tile's next left rows are written
             if (threadIdx.x == 192) {
                 fence_proxy_async_global();

@@ -1,0 +1,54 @@
+"""The stand-alone measurement kernel at the edges of its row groups, row widths and storage formats
+(needs a GB300).  A block takes 4 to 32 rows depending on the row count, rows are written in 16-byte
+pieces with a masked last piece, and FP16 rows are held in registers up to 2048 entries and read twice
+beyond.  Conditionals of every row are compared with the FP64 oracle at the tolerance of the path."""
+import numpy as np
+import pytest
+
+import gen
+import parity
+from oracle import quant
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp32": 1e-5, "bf16x2": 1e-4, "bf16x3l": 1e-4, "fp16x2": 1e-4}
+
+
+def _stored(ts, precision):
+    if precision == "fp32":
+        return ts
+    return [quant.dequant_fp16(A, 1) if precision == "fp16x2" else quant.dequant_bf16(A, 1) for A in ts]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16x2", "bf16x3l", "fp16x2"])
+@pytest.mark.parametrize("d,bonds", [
+    (3, [1, 3, 1, 2, 6, 17, 33, 15, 5, 2, 1]),                # odd and one-entry blocks, next rows of 64 entries
+    (10, [1, 10, 100, 1050, 105, 11, 2, 1]),                  # a row wider than the register-resident path
+    (255, [1, 3, 20, 1]),                                     # the most outcomes a site may have
+])
+def test_measure_edges_against_oracle(precision, d, bonds):
+    import paper_2512_20064_gb300 as F
+
+    b, ts, _ = gen.mps_tensors(len(bonds) - 1, d, max(bonds), base_seed=5, skew=1.5 if d < 255 else None,
+                               dtype=np.complex64, bonds=bonds)
+    N = 37
+    with F.Sampler(precision=precision) as s:
+        s.load_chain(ts)
+        smp, lp, tr = s.sample(b, d, N, 19, trace_rows=N)
+    rep = parity.check(b, _stored(ts, precision), 19, np.arange(N), smp, lp, TOL[precision], dev_trace=tr,
+                       trace_rows=N)
+    assert rep["prob_rows"] == N
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16x2", "fp16x2", "fp8x2"])
+def test_row_groups_give_the_same_bits(precision):
+    """A row's result is the same bits in a call of 12000 rows (32 per block) and in calls of 1 to 6000."""
+    import paper_2512_20064_gb300 as F
+
+    b, ts, _ = gen.mps_tensors(9, 3, 27, base_seed=3, skew=1.5, dtype=np.complex64)
+    with F.Sampler(precision=precision) as s:
+        s.load_chain(ts)
+        smp, lp = s.sample(b, 3, 12000, 4)
+        for n0, N in ((0, 1), (11, 129), (100, 1300), (5, 2600), (1000, 6000)):
+            a, l = s.sample(b, 3, N, 4, n0=n0)
+            assert np.array_equal(a, smp[n0:n0 + N]) and np.array_equal(l, lp[n0:n0 + N])
