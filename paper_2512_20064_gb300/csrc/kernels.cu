@@ -6,6 +6,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "common.cuh"
 #include "launch.h"
 #include "measure.cuh"
@@ -259,10 +262,9 @@ void launch_init_left_f32(float *V, int64_t rows, int ld, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// FP32 SIMT contraction (the plain path): Y = V Bt over a 128 x 128 tile per
-// block, 8 x 8 outputs per thread, K staged 8 at a time in double-buffered
-// shared memory.  Epilogue: store the tile to the FP32 scratch and one sum of
-// squares per row (the tile lies inside one outcome block s).
+// FP32 SIMT contraction (the plain path): Y = V Bt over a (16 TM) x 128 tile per block of 256 threads,
+// TM x 8 outputs per thread.  Epilogue: store the tile to the FP32 scratch and one sum of squares per row
+// (the tile lies inside one outcome block s).
 //
 // Chunked accumulation: each output sums its K = 2 chi_l products in chunks
 // of F32_CHUNK, every chunk in its own FP32 accumulator that is then added to
@@ -272,108 +274,245 @@ void launch_init_left_f32(float *V, int64_t rows, int ld, cudaStream_t st) {
 // random isometries, those errors add up over the sites and surface in the
 // last sites' conditionals; chunks of 64 cut the per-site error about five
 // times (2.3e-5 -> 4.7e-6 at M = 1024, chi = 1024 in a CPU emulation of both
-// orders), at the cost of a second register tile.
+// orders).
+//
+// Bound by the FP32 pipes' operand reads: scalar fma of register operands levels off at 53 TFLOP/s without
+// the totals (two thirds of 152 SMs x 128 lanes, whatever the tile, the lane layout or the shared-memory
+// traffic), 46 with them.  So two outputs of neighbouring rows share one packed fma.rn.f32x2, whose repeated
+// operand (b, b) is read once for TM/2 of them; each half is the correctly rounded fma of its own operands, in
+// the order of a scalar loop.  The running totals live in shared memory, one private column per thread, and
+// are touched once per chunk, so that two blocks fit an SM.  Fragments of the next K entry are loaded while
+// the current ones are multiplied.  32768 rows, K = 512, 2048 columns: 1317 us, 52 TFLOP/s (60 without the
+// totals; scalar, totals in registers, one block per SM: 1447 us).  Keeping every left entry twice in shared
+// memory, to save the register copy of a packed operand, was slower (43 TFLOP/s).
+// A tile whose last 64 columns are padding of its outcome block (2 chi_r <= 64 modulo 128) leaves them out:
+// they are zero, add nothing to the sum of squares, and nothing reads them.
 // ---------------------------------------------------------------------------
-constexpr int F32_BM = 128, F32_BN = 128, F32_BK = 8, F32_THREADS = 256;
-constexpr int F32_CHUNK = 64;  // K entries per partial accumulator (a multiple of F32_BK)
+constexpr int F32_BN = 128, F32_THREADS = 256;
+constexpr int F32_CHUNK = 64;  // K entries per partial accumulator (K is a multiple of it)
 
-__global__ void __launch_bounds__(F32_THREADS, 1)
-contract_f32_kernel(const float *__restrict__ V, int64_t ldV, int64_t row0, const float *__restrict__ Bt, int ldB,
-                    int K, float *__restrict__ Y, int64_t ldY, float *__restrict__ P, int ldP, int rows_valid) {
-    __shared__ __align__(16) float As[2][F32_BK][F32_BM];
-    __shared__ __align__(16) float Bs[2][F32_BK][F32_BN];
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ void fma_f32x2(f32x2 &d, f32x2 a, f32x2 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ f32x2 add_f32x2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 twice_f32x2(float x) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
+    return d;
+}
+__device__ __forceinline__ float2 unpack_f32x2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+}
+
+template <int TM>
+struct F32Tile {
+    static constexpr int BM = 16 * TM;             // rows
+    static constexpr int BK = TM == 8 ? 8 : 16;    // K entries per stage
+    static constexpr int AK = BK * BM / F32_THREADS;  // left entries per thread and stage, along K
+    static constexpr int RG = TM == 8 ? 4 : TM;    // consecutive rows per thread; TM = 8: again 64 rows on
+    static constexpr size_t bytes = sizeof(float) * (2 * BK * (BM + F32_BN) + BM * F32_BN);
+};
+
+// One (16 TM) x (64 NQ) tile.  Thread (ty, tx) holds rows 64 g + RG ty + .. and columns 64 q + 4 tx .. + 3.
+template <int TM, int NQ>
+__device__ __forceinline__ void contract_f32_tile(const float *__restrict__ Ag, int64_t ldV,
+                                                  const float *__restrict__ Bg, int ldB, int K,
+                                                  float *__restrict__ Y, int64_t ldY, float *__restrict__ P, int ldP,
+                                                  int rows_left, float *smem) {
+    using T = F32Tile<TM>;
+    constexpr int BM = T::BM, BK = T::BK, AK = T::AK, RG = T::RG, NP = TM / 2, NC = 4 * NQ;
+    float *As = smem;                                // [2][BK][BM]
+    float *Bs = As + 2 * BK * BM;                    // [2][BK][128]
+    ulonglong2 *tot = reinterpret_cast<ulonglong2 *>(Bs + 2 * BK * F32_BN);  // [NP * NC / 2][threads]
     const int tid = threadIdx.x;
-    const int m0 = blockIdx.y * F32_BM;
-    const int n0 = blockIdx.x * F32_BN;
-    const float *Ag = V + (row0 + m0) * ldV;
-    const int a_row = tid >> 1, a_k = (tid & 1) * 4;
-    const int b_k = tid >> 5, b_n = (tid & 31) * 4;
+    const int a_row = tid % BM, a_k = tid / BM * AK;
+    const int ty = tid >> 4, tx = tid & 15;
+    const float *ap = Ag + (int64_t)a_row * ldV + a_k;
 
-    float4 ra = *reinterpret_cast<const float4 *>(Ag + (int64_t)a_row * ldV + a_k);
-    float4 rb = *reinterpret_cast<const float4 *>(Bt + (int64_t)b_k * ldB + n0 + b_n);
-    As[0][a_k + 0][a_row] = ra.x;
-    As[0][a_k + 1][a_row] = ra.y;
-    As[0][a_k + 2][a_row] = ra.z;
-    As[0][a_k + 3][a_row] = ra.w;
-    *reinterpret_cast<float4 *>(&Bs[0][b_k][b_n]) = rb;
+    float ra[AK];
+    auto load_a = [&](int k0) {
+        if constexpr (AK == 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(ap + k0);
+            ra[0] = v.x, ra[1] = v.y, ra[2] = v.z, ra[3] = v.w;
+        } else {
+            const float2 v = *reinterpret_cast<const float2 *>(ap + k0);
+            ra[0] = v.x, ra[1] = v.y;
+        }
+    };
+    auto store_a = [&](int buf) {
+#pragma unroll
+        for (int e = 0; e < AK; ++e) As[(buf * BK + a_k + e) * BM + a_row] = ra[e];
+    };
+    auto copy_b = [&](int buf, int k0) {
+#pragma unroll
+        for (int id = tid; id < BK * 16 * NQ; id += F32_THREADS) {
+            const int r = id / (16 * NQ), c = id % (16 * NQ) * 4;
+            cp_async16(Bs + (buf * BK + r) * F32_BN + c, Bg + (int64_t)(k0 + r) * ldB + c);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    f32x2 a[2][NP];
+    float b[2][NC];
+    auto load_fragments = [&](int f, int buf, int kk) {
+        const float *A = As + (buf * BK + kk) * BM + ty * RG, *B = Bs + (buf * BK + kk) * F32_BN + tx * 4;
+        if constexpr (RG == 2) {
+            a[f][0] = *reinterpret_cast<const f32x2 *>(A);
+        } else {
+#pragma unroll
+            for (int g = 0; g < TM / RG; ++g) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(A + 64 * g);
+                a[f][2 * g] = v.x;
+                a[f][2 * g + 1] = v.y;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const float4 v = *reinterpret_cast<const float4 *>(B + 64 * q);
+            b[f][4 * q] = v.x, b[f][4 * q + 1] = v.y, b[f][4 * q + 2] = v.z, b[f][4 * q + 3] = v.w;
+        }
+    };
+
+    load_a(0);
+    copy_b(0, 0);
+    store_a(0);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 
-    const int ty = tid >> 4, tx = tid & 15;
-    float acc[8][8], tot[8][8];
+    f32x2 acc[NC][NP];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int j = 0; j < NC; ++j)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            acc[i][j] = 0.f;
-            tot[i][j] = 0.f;
-        }
-
-    const int nk = K / F32_BK;
-    for (int kt = 0; kt < nk; ++kt) {
-        const int cur = kt & 1;
-        if (kt + 1 < nk) {
-            const int k0 = (kt + 1) * F32_BK;
-            ra = *reinterpret_cast<const float4 *>(Ag + (int64_t)a_row * ldV + k0 + a_k);
-            rb = *reinterpret_cast<const float4 *>(Bt + (int64_t)(k0 + b_k) * ldB + n0 + b_n);
-        }
+        for (int i = 0; i < NP; ++i) acc[j][i] = 0ull;
+    load_fragments(0, 0, 0);
+    const int nk = K / BK;
+    for (int k0 = 0; k0 < nk; k0 += F32_CHUNK / BK) {
+#pragma unroll 1
+        for (int kt = k0; kt < k0 + F32_CHUNK / BK; ++kt) {
+            const int cur = kt & 1;
+            if (kt + 1 < nk) {
+                load_a((kt + 1) * BK);
+                copy_b(cur ^ 1, (kt + 1) * BK);
+            }
 #pragma unroll
-        for (int kk = 0; kk < F32_BK; ++kk) {
-            const float4 a0 = *reinterpret_cast<const float4 *>(&As[cur][kk][ty * 4]);
-            const float4 a1 = *reinterpret_cast<const float4 *>(&As[cur][kk][64 + ty * 4]);
-            const float4 b0 = *reinterpret_cast<const float4 *>(&Bs[cur][kk][tx * 4]);
-            const float4 b1 = *reinterpret_cast<const float4 *>(&Bs[cur][kk][64 + tx * 4]);
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        if ((kt + 1) % (F32_CHUNK / F32_BK) == 0 || kt + 1 == nk) {
-            // end of a K chunk: fold its partial sums into the running totals
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    tot[i][j] += acc[i][j];
-                    acc[i][j] = 0.f;
+            for (int kk = 0; kk < BK; ++kk) {
+                if (kk + 1 < BK) {
+                    load_fragments((kk + 1) & 1, cur, kk + 1);
+                } else {
+                    if (kt + 1 < nk) {
+                        store_a(cur ^ 1);
+                        asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    }
+                    __syncthreads();
+                    if (kt + 1 < nk) load_fragments(0, cur ^ 1, 0);
                 }
+#pragma unroll
+                for (int j = 0; j < NC; ++j) {
+                    const f32x2 bb = twice_f32x2(b[kk & 1][j]);
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) fma_f32x2(acc[j][i], a[kk & 1][i], bb);
+                }
+            }
         }
-        if (kt + 1 < nk) {
-            const int nxt = cur ^ 1;
-            As[nxt][a_k + 0][a_row] = ra.x;
-            As[nxt][a_k + 1][a_row] = ra.y;
-            As[nxt][a_k + 2][a_row] = ra.z;
-            As[nxt][a_k + 3][a_row] = ra.w;
-            *reinterpret_cast<float4 *>(&Bs[nxt][b_k][b_n]) = rb;
+        // end of a K chunk: fold its partial sums into the running totals (into acc after the last one),
+        // eight loads in flight
+        const bool first = k0 == 0, last = k0 + F32_CHUNK / BK == nk;
+        constexpr int NE = NP * NC / 2, G = NE < 8 ? NE : 8;
+#pragma unroll
+        for (int e0 = 0; e0 < NE; e0 += G) {
+            if (!first) {
+                ulonglong2 t[G];
+#pragma unroll
+                for (int g = 0; g < G; ++g) t[g] = tot[(e0 + g) * F32_THREADS + tid];
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const int e = 2 * (e0 + g);
+                    acc[e / NP][e % NP] = add_f32x2(t[g].x, acc[e / NP][e % NP]);
+                    acc[(e + 1) / NP][(e + 1) % NP] = add_f32x2(t[g].y, acc[(e + 1) / NP][(e + 1) % NP]);
+                }
+            }
+            if (!last) {
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const int e = 2 * (e0 + g);
+                    tot[(e0 + g) * F32_THREADS + tid] =
+                        make_ulonglong2(acc[e / NP][e % NP], acc[(e + 1) / NP][(e + 1) % NP]);
+                    acc[e / NP][e % NP] = acc[(e + 1) / NP][(e + 1) % NP] = 0ull;
+                }
+            }
         }
-        __syncthreads();
     }
 
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int r = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
-        float ss = 0.f;
+    for (int i = 0; i < TM; ++i) {
+        const int r = 64 * (i / RG) + ty * RG + i % RG;
+        float ss = 0.f, out[NC];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) ss = fmaf(tot[i][j], tot[i][j], ss);
+        for (int j = 0; j < NC; ++j) {
+            const float2 v = unpack_f32x2(acc[j][i / 2]);
+            out[j] = i & 1 ? v.y : v.x;
+            ss = fmaf(out[j], out[j], ss);
+        }
         ss += __shfl_xor_sync(0xffffffffu, ss, 1);
         ss += __shfl_xor_sync(0xffffffffu, ss, 2);
         ss += __shfl_xor_sync(0xffffffffu, ss, 4);
         ss += __shfl_xor_sync(0xffffffffu, ss, 8);
-        if (r < rows_valid) {
-            float *yr = Y + (int64_t)r * ldY + n0;
-            *reinterpret_cast<float4 *>(yr + tx * 4) = make_float4(tot[i][0], tot[i][1], tot[i][2], tot[i][3]);
-            *reinterpret_cast<float4 *>(yr + 64 + tx * 4) = make_float4(tot[i][4], tot[i][5], tot[i][6], tot[i][7]);
-            if (tx == 0) P[(int64_t)r * ldP + blockIdx.x] = ss;
+        if (r < rows_left) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+                *reinterpret_cast<float4 *>(Y + (int64_t)r * ldY + 64 * q + tx * 4) =
+                    make_float4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
+            if (tx == 0) P[(int64_t)r * ldP] = ss;
         }
     }
 }
 
-void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, int64_t rows_pad, const float *Bt,
-                         const SiteLayout &L, const ContractOut &o, cudaStream_t st) {
-    dim3 grid(L.ncols / F32_BN, (unsigned)(rows_pad / F32_BM));
-    contract_f32_kernel<<<grid, F32_THREADS, 0, st>>>(V, ldV, row0, Bt, L.ncols, L.K_pad, o.Y, o.ldY, o.P, o.ldP,
-                                                       o.rows_valid);
+template <int TM>
+__global__ void __launch_bounds__(F32_THREADS, 2)
+contract_f32_kernel(const float *__restrict__ V, int64_t ldV, int64_t row0, const float *__restrict__ Bt, int ldB,
+                    int K, float *__restrict__ Y, int64_t ldY, float *__restrict__ P, int ldP, int rows_valid,
+                    int tiles_per_s, int nreal) {
+    extern __shared__ __align__(16) float f32_smem[];
+    constexpr int BM = F32Tile<TM>::BM;
+    const int64_t m0 = (int64_t)blockIdx.y * BM;
+    const int n0 = blockIdx.x * F32_BN;
+    const int cols = nreal - (int)(blockIdx.x % tiles_per_s) * F32_BN;  // columns of the tile that are not padding
+    const float *Ag = V + (row0 + m0) * ldV;
+    float *Yt = Y + m0 * ldY + n0, *Pt = P + m0 * ldP + blockIdx.x;
+    const int left = rows_valid - (int)m0;
+    if (cols > 64) contract_f32_tile<TM, 2>(Ag, ldV, Bt + n0, ldB, K, Yt, ldY, Pt, ldP, left, f32_smem);
+    else contract_f32_tile<TM, 1>(Ag, ldV, Bt + n0, ldB, K, Yt, ldY, Pt, ldP, left, f32_smem);
+}
+
+void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, const float *Bt, const SiteLayout &L,
+                         const ContractOut &o, cudaStream_t st) {
+    // 128-row tiles, unless 64- or 32-row tiles still fit one per SM: a lone block per SM runs at half the
+    // pace of two, and a shorter tile ends sooner.  Measured, us (128 / 64 / 32 rows): d = 4, chi = 256,
+    // 64 rows: 66 / 39 / 33; 512 rows: 66 / 39 / 58; 1024 rows: 66 / 68 / 109.  128 rows at most, so that no
+    // tile reaches past the left operand's rows (a multiple of 128).
+    const int64_t nx = L.ncols / F32_BN;
+    auto run = [&](auto tm) {
+        using T = F32Tile<decltype(tm)::value>;
+        auto kern = contract_f32_kernel<decltype(tm)::value>;
+        if (T::bytes > 48 * 1024)
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::bytes);
+        const dim3 grid((unsigned)nx, (unsigned)((o.rows_valid + T::BM - 1) / T::BM));
+        kern<<<grid, F32_THREADS, T::bytes, st>>>(V, ldV, row0, Bt, L.ncols, L.K_pad, o.Y, o.ldY, o.P, o.ldP,
+                                                  o.rows_valid, L.tiles_per_s, 2 * L.chi_r);
+    };
+    if (nx * ((o.rows_valid + 31) / 32) <= 152) run(std::integral_constant<int, 2>());
+    else if (nx * ((o.rows_valid + 63) / 64) <= 152) run(std::integral_constant<int, 4>());
+    else run(std::integral_constant<int, 8>());
 }
 
 // ---------------------------------------------------------------------------

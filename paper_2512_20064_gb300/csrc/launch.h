@@ -61,9 +61,9 @@ struct ContractOut {
     int rows_valid;    // rows of this micro-batch
 };
 
-// FP32 SIMT: Y = V[row0 : row0+rows_pad] (ld = ldV, K = L.K_pad) x Bt.
-void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, int64_t rows_pad, const float *Bt,
-                         const SiteLayout &L, const ContractOut &o, cudaStream_t st);
+// FP32 SIMT: Y = V[row0 : row0+o.rows_valid] (ld = ldV, K = L.K_pad) x Bt.  V holds a multiple of 128 rows.
+void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, const float *Bt, const SiteLayout &L,
+                         const ContractOut &o, cudaStream_t st);
 
 // tcgen05 BF16 split-precision contraction.  tmA[p] / tmB[p] are tensor maps
 // over the operand planes (a_planes in {1,2,3}, b_planes in {1,2}); the

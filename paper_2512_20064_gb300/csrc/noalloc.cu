@@ -213,7 +213,7 @@ extern "C" int fastmps_sample_noalloc(fastmps_handle h, int M, int d, const int 
                 e = launch_contract_tc(ta, L, co, hv.num_sms, d_err, st);
                 if (e != cudaSuccess) return set_error(h, FASTMPS_ERR_CUDA, "contraction launch failed");
             } else {
-                launch_contract_f32(V32[cur], ldV, r0, roundup(rows, 128), sv.Bt, L, co, st);
+                launch_contract_f32(V32[cur], ldV, r0, sv.Bt, L, co, st);
             }
             MeasureArgs ma;
             ma.Y = Y;
