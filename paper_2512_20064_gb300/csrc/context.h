@@ -107,6 +107,7 @@ struct fastmps_ctx {
     fastmps::DevBuf disp_io;  // device staging of fastmps_displacement's host inputs / outputs
     fastmps::DevBuf trunc;    // device gather of the leading block of a truncated Vidal-form site
     fastmps::DevBuf disp_tab; // constants of the displacement entries for dimension disp_tab_d
+    fastmps::DevBuf chain_sites;  // site table of an FP32 call that runs in one launch
     fastmps::DevBuf disp_D, disp_u;  // per-row matrices and uniforms of one displaced micro-batch
     int disp_tab_d = 0;
     std::vector<float> disp_tab_host;

@@ -14,6 +14,8 @@ namespace fastmps {
 
 namespace {
 
+constexpr size_t kChainSmemLimit = 232448;  // 227 KB: the most shared memory a block may have
+
 struct EventTimer {
     fastmps_handle h;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> contract, measure, copy;
@@ -37,6 +39,86 @@ struct EventTimer {
         return s;
     }
 };
+
+// Host copies of the outputs (from the staging buffers), the error word and the call's statistics; waits for
+// the call's work.  trace_host: null where the trace was written in place.
+int finish_call(fastmps_handle h, EventTimer &timer, std::chrono::steady_clock::time_point t_start,
+                uint8_t *out_samples, bool samples_dev, double *out_logprob, bool logp_dev, double *trace_host,
+                const double *trace_buf, int M, int d, int64_t N, int64_t trace_rows) {
+    cudaStream_t st = h->stream;
+    cudaError_t e;
+    if (out_samples && !samples_dev) {
+        e = cudaMemcpyAsync(out_samples, h->Dout.p, (size_t)N * M, cudaMemcpyDeviceToHost, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "copy of samples");
+        h->stats.d2h_bytes += (int64_t)N * M;
+    }
+    if (out_logprob && !logp_dev) {
+        e = cudaMemcpyAsync(out_logprob, h->logp.p, (size_t)N * 8, cudaMemcpyDeviceToHost, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "copy of log-probabilities");
+        h->stats.d2h_bytes += N * 8;
+    }
+    if (trace_host && trace_buf) {
+        e = cudaMemcpyAsync(trace_host, trace_buf, (size_t)M * trace_rows * d * 8, cudaMemcpyDeviceToHost, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "copy of trace");
+    }
+    int herr = 0;
+    e = cudaMemcpyAsync(&herr, h->err.p, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e != cudaSuccess) return cuda_fail(h, e, "copy of error word");
+    e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(h, e, "sampling");
+    h->stats.ms_contract = timer.total(timer.contract);
+    h->stats.ms_measure = timer.total(timer.measure);
+    h->stats.ms_h2d = timer.total(timer.copy);
+    h->stats.ms_total =
+        std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
+    if (herr == kDevNumeric)
+        return fail(h, FASTMPS_ERR_NUMERIC, "a sample's probabilities summed to zero or a non-finite value");
+    if (herr != 0)
+        return fail(h, FASTMPS_ERR_TIMEOUT,
+                    "a bounded device wait in the contraction kernel gave up (code " + std::to_string(herr) + ")");
+    return FASTMPS_OK;
+}
+
+// FP32 calls that run in one launch (launch_chain_f32): the site table and the block's shared-memory extents.
+struct ChainPlan {
+    std::vector<ChainSite> sites;
+    int k_max = 0, y_ld = 0, p_ld = 0;
+};
+
+// Whether an FP32 call runs in one launch: if its estimated time is well below that of two launches per site.
+// Both sides in microseconds, fitted to measurements (24-site chains, 1 to 131072 rows, d = 2..6, chi = 8..256):
+//   one launch:  per wave of blocks (three per SM, fewer where shared memory says so) and site 3.6, plus 0.67
+//                for each stage of 16 K-entries x 128 columns;
+//   two launches: 22 per site (two launches, an event each way), plus the products at 52 TFLOP/s on whole
+//                64-column halves, the scratch, selected and next rows at 5 TB/s, and the FP64 draws.
+// E.g. d = 2, chi = 32: 64 rows 151 against 584 us, 131072 rows 1731 against 2407; d = 4, chi = 64: 4864 rows
+// 645 against 866, 10000 rows 1852 against 1376 (two launches); chi = 128 and up: two launches.  Where the two
+// estimates are close the two-launch path stays (the factor 0.8: d = 6, chi = 90, 4864 rows 2160 against 1800).
+bool chain_plan(const std::vector<Tensor *> &ts, int d, int64_t N, int num_sms, ChainPlan *c) {
+    c->sites.clear();
+    double one = 0.0, two = 0.0;  // one: per wave of blocks
+    for (const Tensor *t : ts) {
+        ChainSite s;
+        s.Bt = t->Bt.as<float>();
+        s.ldB = t->L.ncols;
+        s.K = (int)roundup(2 * (int64_t)t->L.chi_l, 16);
+        s.nreal = 2 * t->L.chi_r;
+        s.tiles_per_s = t->L.tiles_per_s;
+        c->sites.push_back(s);
+        c->k_max = std::max(c->k_max, s.K);
+        c->y_ld = std::max(c->y_ld, d * (int)roundup(s.nreal, 4));
+        c->p_ld = std::max(c->p_ld, d * s.tiles_per_s);
+        if (c->k_max > 1024 || c->y_ld > 2048) return false;  // wider than a block's shared memory
+        one += 3.6 + 0.67 * (s.K / 16) * std::ceil(d * (double)roundup(s.nreal, 16) / 128.0);
+        two += 22.0 + (double)N * (1.9e-4 + (double)t->L.K_pad * d * (double)roundup(s.nreal, 64) / 26e6 +
+                                   4.0 * ((d + 2.0) * s.nreal + s.nreal) / 5e6);
+    }
+    const size_t smem = chain_f32_smem(c->k_max, c->y_ld, c->p_ld, d);
+    if (smem > kChainSmemLimit) return false;
+    const int64_t per_sm = std::min<int64_t>(kChainBlocksPerSm, (int64_t)(kChainSmemLimit / (smem + 1024)));
+    const int64_t slots = std::max<int64_t>(1, per_sm) * num_sms;
+    return (double)((chain_f32_blocks(N) + slots - 1) / slots) * one < 0.8 * two;
+}
 
 }  // namespace
 
@@ -99,6 +181,8 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
     if (N == 0) return FASTMPS_OK;
     const bool stream_mode = h->opt.residency == FASTMPS_HOST_STREAM;
     const bool bf16 = is_bf16(h);
+    ChainPlan chain;
+    const bool in_one_launch = !bf16 && !mu_dev && chain_plan(ts, d, N, h->num_sms, &chain);
     cudaStream_t st = h->stream;
     cudaError_t e;
 
@@ -131,7 +215,7 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
     const int planes = bf16 ? plan.a_planes : 1;
     const size_t elem = fp8 ? 1 : (bf16 ? 2 : 4);
     if (fp8) ldV = (int)roundup(ldV, 128);
-    for (int x = 0; x < 2; ++x)
+    for (int x = 0; x < 2 && !in_one_launch; ++x)
         for (int p = 0; p < planes; ++p)
             if (!h->V[x][p].ensure((size_t)N_pad * ldV * elem))
                 return fail(h, FASTMPS_ERR_OOM, "left-operand allocation failed");
@@ -139,11 +223,12 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
     const bool fused = bf16 && !fp8 && h->opt.fused_measure == 1 && !mu_dev;
     const int nybuf = (J > 1 && !fused) ? 2 : 1;
 
-    if (ncols_max > 0)
+    if (ncols_max > 0 && !in_one_launch)
         for (int b = 0; b < nybuf; ++b)
             if (!h->Y[b].ensure((size_t)N2 * ncols_max * 4) || !h->P[b].ensure((size_t)N2 * ldP_max * 4))
                 return fail(h, FASTMPS_ERR_OOM, "scratch allocation failed");
-    if (!h->logp.ensure((size_t)N_pad * 8) || !h->O.ensure((size_t)M * N_pad) || !h->err.ensure(sizeof(int)))
+    if (!h->logp.ensure((size_t)N_pad * 8) || (!in_one_launch && !h->O.ensure((size_t)M * N_pad)) ||
+        !h->err.ensure(sizeof(int)))
         return fail(h, FASTMPS_ERR_OOM, "work-buffer allocation failed");
     const bool samples_dev = is_device_ptr(out_samples);
     const bool logp_dev = is_device_ptr(out_logprob);
@@ -193,6 +278,40 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
     int *d_err = h->err.as<int>();
     e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
     if (e != cudaSuccess) return cuda_fail(h, e, "memset");
+    EventTimer timer(h);
+    if (in_one_launch) {
+        if (!h->chain_sites.ensure(chain.sites.size() * sizeof(ChainSite)))
+            return fail(h, FASTMPS_ERR_OOM, "work-buffer allocation failed");
+        e = cudaMemcpyAsync(h->chain_sites.p, chain.sites.data(), chain.sites.size() * sizeof(ChainSite),
+                            cudaMemcpyHostToDevice, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "copy of the site table");
+        ChainArgs ca;
+        ca.sites = h->chain_sites.as<ChainSite>();
+        ca.M = M;
+        ca.d = d;
+        ca.k_max = chain.k_max;
+        ca.y_ld = chain.y_ld;
+        ca.p_ld = chain.p_ld;
+        ca.rows = N;
+        ca.seed = seed;
+        ca.n0 = (uint64_t)n0;
+        ca.job = job;
+        ca.samples = !out_samples ? nullptr : samples_dev ? out_samples : h->Dout.as<uint8_t>();
+        ca.logp = !out_logprob ? nullptr : logp_dev ? out_logprob : h->logp.as<double>();
+        ca.trace = trace_buf;
+        ca.trace_rows = trace_rows;
+        ca.trace_slot = trace_slot;
+        ca.err = d_err;
+        cudaEvent_t c0 = timer.get(), c1 = timer.get();
+        cudaEventRecord(c0, st);
+        e = launch_chain_f32(ca, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "chain launch");
+        cudaEventRecord(c1, st);
+        timer.contract.push_back({c0, c1});
+        h->stats.launches = h->stats.contract_launches = 1;
+        return finish_call(h, timer, t_start, out_samples, samples_dev, out_logprob, logp_dev,
+                           trace_dev ? nullptr : trace_probs, trace_buf, M, d, N, trace_rows);
+    }
     cudaMemsetAsync(h->logp.p, 0, (size_t)N_pad * 8, st);
     __nv_bfloat16 *Vp[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
     for (int x = 0; x < 2; ++x)
@@ -208,7 +327,6 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
         launch_init_left_f32(h->V[0][0].as<float>(), N_pad, ldV, st);
     h->stats.launches += 1;
 
-    EventTimer timer(h);
     cudaStream_t ms = h->measure_stream;
     int64_t g = 0;  // micro-batch counter over the whole call
     int64_t last_measured = -1;  // micro-batch whose measurement ran last on the measurement stream
@@ -424,38 +542,13 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
         uint8_t *dst = samples_dev ? out_samples : h->Dout.as<uint8_t>();
         launch_transpose_outcomes(h->O.as<uint8_t>(), N_pad, N, M, dst, st);
         h->stats.launches += 1;
-        if (!samples_dev) {
-            e = cudaMemcpyAsync(out_samples, dst, (size_t)N * M, cudaMemcpyDeviceToHost, st);
-            if (e != cudaSuccess) return cuda_fail(h, e, "copy of samples");
-            h->stats.d2h_bytes += (int64_t)N * M;
-        }
     }
-    if (out_logprob) {
-        e = cudaMemcpyAsync(out_logprob, h->logp.p, (size_t)N * 8,
-                            logp_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
+    if (out_logprob && logp_dev) {
+        e = cudaMemcpyAsync(out_logprob, h->logp.p, (size_t)N * 8, cudaMemcpyDeviceToDevice, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "copy of log-probabilities");
-        if (!logp_dev) h->stats.d2h_bytes += N * 8;
     }
-    if (trace_buf && !trace_dev) {
-        e = cudaMemcpyAsync(trace_probs, trace_buf, (size_t)M * trace_rows * d * 8, cudaMemcpyDeviceToHost, st);
-        if (e != cudaSuccess) return cuda_fail(h, e, "copy of trace");
-    }
-    int herr = 0;
-    e = cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "copy of error word");
-    e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "sampling");
-    h->stats.ms_contract = timer.total(timer.contract);
-    h->stats.ms_measure = timer.total(timer.measure);
-    h->stats.ms_h2d = timer.total(timer.copy);
-    h->stats.ms_total =
-        std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
-    if (herr == kDevNumeric)
-        return fail(h, FASTMPS_ERR_NUMERIC, "a sample's probabilities summed to zero or a non-finite value");
-    if (herr != 0)
-        return fail(h, FASTMPS_ERR_TIMEOUT,
-                    "a bounded device wait in the contraction kernel gave up (code " + std::to_string(herr) + ")");
-    return FASTMPS_OK;
+    return finish_call(h, timer, t_start, out_samples, samples_dev, out_logprob, logp_dev,
+                       trace_dev ? nullptr : trace_probs, trace_buf, M, d, N, trace_rows);
 }
 
 }  // namespace fastmps

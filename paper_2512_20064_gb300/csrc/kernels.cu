@@ -10,6 +10,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "f32x2.cuh"
 #include "launch.h"
 #include "measure.cuh"
 
@@ -289,31 +290,7 @@ void launch_init_left_f32(float *V, int64_t rows, int ld, cudaStream_t st) {
 // they are zero, add nothing to the sum of squares, and nothing reads them.
 // ---------------------------------------------------------------------------
 constexpr int F32_BN = 128, F32_THREADS = 256;
-constexpr int F32_CHUNK = 64;  // K entries per partial accumulator (K is a multiple of it)
-
-typedef unsigned long long f32x2;
-
-__device__ __forceinline__ void fma_f32x2(f32x2 &d, f32x2 a, f32x2 b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ f32x2 add_f32x2(f32x2 a, f32x2 b) {
-    f32x2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f32x2 twice_f32x2(float x) {
-    f32x2 d;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
-    return d;
-}
-__device__ __forceinline__ float2 unpack_f32x2(f32x2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
-}
+constexpr int F32_CHUNK = kF32Chunk;  // K is a multiple of it
 
 template <int TM>
 struct F32Tile {
@@ -360,7 +337,7 @@ __device__ __forceinline__ void contract_f32_tile(const float *__restrict__ Ag, 
             const int r = id / (16 * NQ), c = id % (16 * NQ) * 4;
             cp_async16(Bs + (buf * BK + r) * F32_BN + c, Bg + (int64_t)(k0 + r) * ldB + c);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        cp_async_commit();
     };
     f32x2 a[2][NP];
     float b[2][NC];
@@ -386,7 +363,7 @@ __device__ __forceinline__ void contract_f32_tile(const float *__restrict__ Ag, 
     load_a(0);
     copy_b(0, 0);
     store_a(0);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    cp_async_wait<0>();
     __syncthreads();
 
     f32x2 acc[NC][NP];
@@ -411,7 +388,7 @@ __device__ __forceinline__ void contract_f32_tile(const float *__restrict__ Ag, 
                 } else {
                     if (kt + 1 < nk) {
                         store_a(cur ^ 1);
-                        asm volatile("cp.async.wait_group 0;" ::: "memory");
+                        cp_async_wait<0>();
                     }
                     __syncthreads();
                     if (kt + 1 < nk) load_fragments(0, cur ^ 1, 0);

@@ -65,6 +65,33 @@ struct ContractOut {
 void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, const float *Bt, const SiteLayout &L,
                          const ContractOut &o, cudaStream_t st);
 
+// FP32, a whole chain in one launch (chain.cu).  sites: device table; y_ld >= d * roundup(2 chi_r, 4) and a
+// multiple of 4, p_ld >= d * tiles_per_s, k_max >= K of every site.
+struct ChainSite {
+    const float *Bt;  // [K_pad][ldB]
+    int ldB;
+    int K;            // 2 chi_l rounded up to 16
+    int nreal;        // 2 chi_r
+    int tiles_per_s;  // 128-column tiles per outcome block
+};
+struct ChainArgs {
+    const ChainSite *sites;
+    int M, d, k_max, y_ld, p_ld;
+    int64_t rows;
+    uint64_t seed, n0;
+    uint32_t job;
+    uint8_t *samples;       // device [rows][M] or null
+    double *logp;           // device [rows] or null
+    double *trace;          // device [M][trace_rows][d] or null
+    int64_t trace_rows;
+    const int *trace_slot;  // device, per row, or null (rows 0 .. trace_rows-1)
+    int *err;
+};
+constexpr int kChainBlocksPerSm = 3;  // as far as registers go
+size_t chain_f32_smem(int k_max, int y_ld, int p_ld, int d);
+int64_t chain_f32_blocks(int64_t rows);
+cudaError_t launch_chain_f32(const ChainArgs &a, cudaStream_t st);
+
 // tcgen05 BF16 split-precision contraction.  tmA[p] / tmB[p] are tensor maps
 // over the operand planes (a_planes in {1,2,3}, b_planes in {1,2}); the
 // products accumulated are (prod_a[q], prod_b[q]) for q < nprod.
