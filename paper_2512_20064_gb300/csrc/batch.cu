@@ -338,8 +338,9 @@ extern "C" int fastmps_sample_batch(fastmps_handle runner, int count, const fast
                 ++si;
             }
         }
-        // counters: [0, 2) task queue (64-bit), then measured[slot], then tiles_done[segment m-tile]
-        const size_t counter_ints = 4 + (size_t)slot_base[count] + (size_t)done;
+        // counters: [0, 2) task queue, [2, 4) measurement queue (64-bit each), [4] length of the measurement
+        // list, then from 8 the list (64-bit entries), measured[slot], tiles_done[segment m-tile]
+        const size_t counter_ints = 8 + 2 * (size_t)done + (size_t)slot_base[count] + (size_t)done;
         if (!bs->counters.ensure(counter_ints * sizeof(int)))
             return set_error(runner, FASTMPS_ERR_OOM, "counter allocation failed");
         e = cudaMemcpyAsync(bs->segs_dev.p, hs, total_segs * sizeof(PSegment), cudaMemcpyHostToDevice, st);
@@ -383,9 +384,13 @@ extern "C" int fastmps_sample_batch(fastmps_handle runner, int count, const fast
         g.nseg = (int)total_segs;
         g.total_tasks = task;
         int *ctr = bs->counters.as<int>();
+        g.total_m_tiles = done;
         g.queue = ctr;
-        g.measured = ctr + 4;
-        g.tiles_done = ctr + 4 + slot_base[count];
+        g.measure_queue = ctr + 2;
+        g.ready_tail = ctr + 4;
+        g.ready = ctr + 8;
+        g.measured = ctr + 8 + 2 * done;
+        g.tiles_done = g.measured + slot_base[count];
         g.a_planes = a_planes;
         g.b_planes = b_planes;
         g.nprod = nprod;

@@ -526,35 +526,23 @@ __global__ void __launch_bounds__(MEASURE_THREADS) measure_kernel(const MeasureA
     __syncthreads();
     double Z = 0.0, ws = 0.0;
     bool ok = false;
+    const RowSums w{w_sh + tid * d, nullptr, d, T};
     if (tid < count) {
-        const double *w = w_sh + tid * d;
-        for (int s = 0; s < d; ++s) Z += w[s];
-        const double t = u * Z;
-        double C = 0.0;
-        int sstar = d - 1;
-        for (int s = 0; s < d; ++s) {
-            C += w[s];
-            if (s == d - 1 || C >= t) {
-                sstar = s;
-                ws = w[s];
-                break;
-            }
-        }
-        ok = (Z > 0.0) && isfinite(Z) && (ws > 0.0);
+        const int sstar = draw_row(w, u, &Z, &ws, &ok);
         sstar_sh[tid] = sstar;
         scale_sh[tid] = ok ? rsqrtf((float)ws) : 0.f;
         a.outcomes[r0 + tid] = (uint8_t)sstar;
     }
     __syncthreads();
     if constexpr (!kScaled) {
-        write_rows_flat(a, tid, MEASURE_THREADS, r0, count, sstar_sh, scale_sh);
+        write_rows_flat<1>(a, tid, MEASURE_THREADS, r0, count, sstar_sh, scale_sh);
     } else {
         for (int j = tid >> 5; j < count; j += MEASURE_THREADS / 32)
             write_row_scaled(a, lane, a.Y + (int64_t)(r0 + j) * a.ldY + (int64_t)sstar_sh[j] * a.Cs, scale_sh[j],
                              a.row0 + r0 + j);
     }
     // nothing waits for the logarithm: it follows the row writes
-    if (tid < count) measure_finish(a, r0 + tid, ws, Z, ok, lp, w_sh + tid * d);
+    if (tid < count) measure_finish(a, r0 + tid, ws, Z, ok, lp, w);
 }
 
 void launch_measure(const MeasureArgs &a, cudaStream_t st) {

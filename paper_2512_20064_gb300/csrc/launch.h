@@ -207,8 +207,8 @@ struct PSegment {  // 64-byte aligned through its CUtensorMap members
     int num_m_tiles, num_n_tiles, num_k_blocks, bn;
     uint32_t idesc, tx_bytes;
     int row0;            // TMA y coordinate of the chunk's first row in the job's left-operand buffers
-    int step;            // c * M + k: measurements every m-tile of this chunk has had before this segment
-    int64_t slot_base;   // measured[slot_base + mt]: measurements completed by m-tile slot mt of the job
+    int step;            // c * M + k: steps every m-tile of this chunk has been measured for before this segment
+    int64_t slot_base;   // measured[slot_base + mt]: 32-row measurements completed by m-tile slot mt of the job
     int64_t done_base;   // tiles_done[done_base + mt]: finished tiles of m-tile mt of this segment
     float *Y;
     int64_t ldY;
@@ -222,7 +222,11 @@ struct PersistentArgs {
     const MeasureArgs *meas;   // device, one per segment
     int nseg;
     int64_t total_tasks;
-    int *queue;                // device: next task (zero at launch)
+    int64_t total_m_tiles;     // of all segments
+    int *queue;                // device: next task, 64 bits (zero at launch)
+    int *measure_queue;        // device: next measurement, 64 bits (zero at launch)
+    int *ready_tail;           // device: m-tiles put on the measurement list (zero at launch)
+    int *ready;                // device: the list, 64 bits per segment m-tile (zero at launch)
     int *measured;             // device: per job m-tile slot (zero at launch)
     int *tiles_done;           // device: per segment m-tile (zero at launch)
     int a_planes, b_planes, nprod;

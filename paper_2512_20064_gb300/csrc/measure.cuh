@@ -14,7 +14,7 @@ namespace fastmps {
 
 // ---------------------------------------------------------------------------
 // Measurement (Algorithm 2 with the exact per-sample rescaling of Sec. 3.3.1).
-// Phase 1, one thread per sample (measure_draw):
+// Phase 1, one thread per sample (draw_row, measure_finish):
 //  * w_s = sum of the FP32 per-tile sums of squares of outcome block s,
 //    accumulated in FP64;
 //  * C_s = w_0 + ... + w_s in s order (FP64), Z = C_{d-1}, Philox uniform u,
@@ -86,11 +86,13 @@ __device__ __forceinline__ void store_row8(const MeasureArgs &a, int64_t off, co
 }
 
 // Next left rows of micro-batch rows r0 .. r0+count-1 (FP32 or BF16 planes) by `nt` threads: the rows'
-// 8-entry pieces are dealt to the threads in order, so threads stay busy whether rows are 64 or 4096
-// entries wide.  sstar, scale: per row.  Pieces of 8 entries make every load 32 bytes and every BF16
-// plane store 16 bytes; more in flight per thread costs registers, so resident warps, and gains nothing.
-// 131072 rows of 512 entries (measurement kernel, 32 rows per block): 94 us with one 8-entry piece at a
-// time, 98 us with two, 137 us with four of 4 entries (16-byte loads, 8-byte stores).
+// 8-entry pieces are dealt to the threads in order, U of them in flight per thread, so threads stay busy
+// whether rows are 64 or 4096 entries wide.  sstar, scale: per row.  Pieces of 8 entries make every load 32
+// bytes and every BF16 plane store 16 bytes.
+// U = 1 where many blocks share an SM: more in flight per thread costs registers, so resident warps, and
+// gains nothing (131072 rows of 512 entries, 32 rows per block: 94 us, 98 with two; 137 us with four pieces
+// of 4 entries).  U = 8 where four warps are all an SM has for the measurement.
+template <int U>
 __device__ __forceinline__ void write_rows_flat(const MeasureArgs &a, int tid, int nt, int r0, int count,
                                                 const int *sstar, const float *scale) {
     const int nreal = 2 * a.chi_r;
@@ -98,13 +100,25 @@ __device__ __forceinline__ void write_rows_flat(const MeasureArgs &a, int tid, i
     const int step_r = nt / per_row, step_c = nt - step_r * per_row;
     int r = tid / per_row, c = tid - r * per_row;
     while (r < count) {
-        const Entries8 v = load_block8(a.Y + (int64_t)(r0 + r) * a.ldY + (int64_t)sstar[r] * a.Cs, 8 * c, nreal);
-        store_row8(a, (a.row0 + r0 + r) * (int64_t)a.ld_next + 8 * c, v, scale[r]);
-        r += step_r;
-        c += step_c;
-        if (c >= per_row) {
-            c -= per_row;
-            ++r;
+        Entries8 v[U];
+        int rr[U], cc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            rr[u] = r;
+            cc[u] = 8 * c;
+            if (r < count)
+                v[u] = load_block8(a.Y + (int64_t)(r0 + r) * a.ldY + (int64_t)sstar[r] * a.Cs, 8 * c, nreal);
+            r += step_r;
+            c += step_c;
+            if (c >= per_row) {
+                c -= per_row;
+                ++r;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (rr[u] >= count) break;
+            store_row8(a, (a.row0 + r0 + rr[u]) * (int64_t)a.ld_next + cc[u], v[u], scale[rr[u]]);
         }
     }
 }
@@ -196,81 +210,115 @@ __device__ __forceinline__ void measure_write_rows(const MeasureArgs &a, int tid
                                 a.row0 + r0 + j);
         return;
     }
-    write_rows_flat(a, tid, nt, r0, count, sstar, scale);
+    write_rows_flat<8>(a, tid, nt, r0, count, sstar, scale);
 }
 
 // w_s of one row: the FP64 sum, in tile order, of its T per-tile sums of squares.  P is read through L2
-// (it may have been written by other thread blocks of the same kernel); eight loads are in flight.
+// (it may have been written by other thread blocks of the same kernel), eight loads in flight.
 __device__ __forceinline__ double sum_tiles(const float *P, int T) {
     double acc = 0.0;
-    int j = 0;
-    for (; j + 8 <= T; j += 8) {
+    for (int j = 0; j < T; j += 8) {
         float x[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = __ldcg(P + j + e);
+        for (int e = 0; e < 8; ++e) x[e] = j + e < T ? __ldcg(P + j + e) : 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc += (double)x[e];
+        for (int e = 0; e < 8; ++e)
+            if (j + e < T) acc += (double)x[e];
     }
-    for (; j < T; ++j) acc += (double)__ldcg(P + j);
     return acc;
 }
 
-// Log-probability, numeric check and optional trace of one drawn row (w: its d sums, Z their total).
+// Calls f(s, w_s) for s = 0 .. d-1 until it returns true, the sums as in sum_tiles.  The d T values of a row are
+// contiguous: 16 loads in flight, whatever T is (one thread has the whole row, and each load takes most of a
+// microsecond).
+template <class F>
+__device__ __forceinline__ void each_outcome_sum(const float *P, int d, int T, F f) {
+    const int n = d * T;
+    double acc = 0.0;
+    int s = 0, left = T;
+    for (int j = 0; j < n; j += 16) {
+        float x[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = j + e < n ? __ldcg(P + j + e) : 0.f;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            if (j + e >= n) break;
+            acc += (double)x[e];
+            if (--left == 0) {
+                if (f(s, acc)) return;
+                acc = 0.0;
+                left = T;
+                ++s;
+            }
+        }
+    }
+}
+
+// The sums w_s of one row: in shared memory (w), or still as per-tile sums in P.
+struct RowSums {
+    const double *w;
+    const float *P;
+    int d, T;
+    template <class F>
+    __device__ __forceinline__ void each(F f) const {
+        if (w) {
+            for (int s = 0; s < d; ++s)
+                if (f(s, w[s])) return;
+        } else {
+            each_outcome_sum(P, d, T, f);
+        }
+    }
+};
+
+// The draw of one row (FP64, in s order): Z = w_0 + ... + w_{d-1}; s* is the first s < d-1 with
+// C_s >= u Z (else d-1), which equals #{s < d-1 : C_s < u Z} because C is non-decreasing.
+__device__ __forceinline__ int draw_row(const RowSums &row, double u, double *Z_out, double *ws_out, bool *ok_out) {
+    double Z = 0.0;
+    row.each([&](int, double w) {
+        Z += w;
+        return false;
+    });
+    const double t = u * Z;
+    double C = 0.0, ws = 0.0;
+    int sstar = row.d - 1;
+    row.each([&](int s, double w) {
+        C += w;
+        if (s < row.d - 1 && !(C >= t)) return false;
+        sstar = s;
+        ws = w;
+        return true;
+    });
+    *Z_out = Z;
+    *ws_out = ws;
+    *ok_out = (Z > 0.0) && isfinite(Z) && (ws > 0.0);
+    return sstar;
+}
+
+// Log-probability, numeric check and optional trace of one drawn row.
 __device__ __forceinline__ void measure_finish(const MeasureArgs &a, int row, double ws, double Z, bool ok, double lp,
-                                               const double *w) {
+                                               const RowSums &w) {
     const int64_t grow = a.row0 + row;
     if (ok) a.logp[grow] = lp + log(ws / Z);
     else atomicExch(a.err, (int)kDevNumeric);
     const int64_t slot = a.trace ? (a.trace_slot ? (int64_t)a.trace_slot[grow] : (grow < a.trace_rows ? grow : -1))
                                  : -1;
     if (slot >= 0)
-        for (int s = 0; s < a.d; ++s) a.trace[slot * a.d + s] = ok ? w[s] / Z : 0.0;
+        w.each([&](int s, double x) {
+            a.trace[slot * a.d + s] = ok ? x / Z : 0.0;
+            return false;
+        });
 }
 
-// Phase 1 for sample `row` of the micro-batch (row < a.rows): draw, outcome,
-// log-probability, optional trace.  Returns the outcome and sets *scale to
-// 1/sqrt(w_{s*}).  P is read through L2 (it may have been written by other
-// thread blocks of the same kernel).
+// Phase 1 for sample `row` of the micro-batch (row < a.rows) by one thread: draw, outcome,
+// log-probability, optional trace.  Returns the outcome and sets *scale to 1/sqrt(w_{s*}).
 __device__ __forceinline__ int measure_draw(const MeasureArgs &a, int row, float *scale_out) {
-    int sstar = 0;
-    float scale = 0.f;
-    {
-        const float *Prow = a.P + (int64_t)row * a.ldP;
-        const int T = a.tiles_per_s;
-        // pass 1: Z = w_0 + ... + w_{d-1} in s order
-        double Z = 0.0;
-        for (int s = 0; s < a.d; ++s) Z += sum_tiles(Prow + s * T, T);
-        const uint64_t n = a.n_base + (uint64_t)row;
-        const double t = sample_uniform(a.seed, n, a.k, a.job) * Z;
-        // pass 2: the same partial sums again; s* is the first s < d-1 with C_s >= t (else d-1),
-        // which equals #{s < d-1 : C_s < t} because C is non-decreasing
-        double C = 0.0, ws = 0.0;
-        sstar = a.d - 1;
-        for (int s = 0; s < a.d; ++s) {
-            const double acc = sum_tiles(Prow + s * T, T);
-            C += acc;
-            if (s == a.d - 1 || C >= t) {
-                sstar = s;
-                ws = acc;
-                break;
-            }
-        }
-        const bool ok = (Z > 0.0) && isfinite(Z) && (ws > 0.0);
-        const int64_t grow = a.row0 + row;
-        a.outcomes[row] = (uint8_t)sstar;
-        if (ok) a.logp[grow] += log(ws / Z);
-        else atomicExch(a.err, (int)kDevNumeric);
-        const int64_t slot = a.trace ? (a.trace_slot ? (int64_t)a.trace_slot[grow] : (grow < a.trace_rows ? grow : -1))
-                                     : -1;
-        if (slot >= 0) {
-            for (int s = 0; s < a.d; ++s) {
-                const double acc = sum_tiles(Prow + s * T, T);
-                a.trace[slot * a.d + s] = ok ? acc / Z : 0.0;
-            }
-        }
-        scale = ok ? rsqrtf((float)ws) : 0.f;
-    }
-    *scale_out = scale;
+    const RowSums w{nullptr, a.P + (int64_t)row * a.ldP, a.d, a.tiles_per_s};
+    double Z, ws;
+    bool ok;
+    const int sstar = draw_row(w, sample_uniform(a.seed, a.n_base + (uint64_t)row, a.k, a.job), &Z, &ws, &ok);
+    a.outcomes[row] = (uint8_t)sstar;
+    measure_finish(a, row, ws, Z, ok, a.logp[a.row0 + row], w);
+    *scale_out = ok ? rsqrtf((float)ws) : 0.f;
     return sstar;
 }
 

@@ -55,15 +55,26 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity) 
 // site k are written by the measurement of site k-1, and the chunk's scratch
 // rows are free once the previous step's measurement has read them).  The
 // epilogue stores the FP32 tile and its sums of squares and counts the finished
-// tiles of the m-tile; the block that finishes the last one hands the m-tile to
-// its four measurement warps, which draw, write the next left rows (Algorithm 2)
-// and release the slot's counter.  Warps: 0 TMA producer, 1 MMA issuer, 2-5
-// epilogue, 6-9 measurement (320 threads).
+// tiles of the m-tile; the thread that counts the last one publishes the m-tile
+// in the launch's measurement list.  Measurements are handed out like tasks: each
+// group of four measurement warps takes the next 32 rows of the list from a global
+// counter, in the order of publication, waits (bounded) for them to be published,
+// draws, writes the next left rows (Algorithm 2) and adds one to the slot's counter,
+// which stands at kMeasureParts for every step measured.  Warps: 0 TMA producer,
+// 1 MMA issuer, 2-5 epilogue, 6-13 two measurement groups (448 threads).
+//
+// The list is what keeps a step short: the steps of a chain follow each other, and
+// each takes as long as its slowest m-tile.  When the block that finished an m-tile's
+// last tile also measured all of it (128 rows, 43 us), some block had several m-tiles
+// waiting in every round and a round of 226 m-tiles took 200 us on 152 blocks.
 // ===========================================================================
-constexpr int kPThreads = 320;
+constexpr int kPThreads = 448;
 constexpr int kTaskRing = 16;
-constexpr int kMRing = 4;
 constexpr int kPBarrierBytes = 3072;
+constexpr int kMeasureParts = 4;                   // measurements of an m-tile: 32 rows each
+constexpr int kMeasureGroups = 2;                  // groups of four warps per block
+constexpr int kMeasureSums = 1024;                 // (row, outcome) sums of a group in shared memory
+constexpr int kPMeasureBytes = kMeasureGroups * kMeasureSums * 8;
 
 struct PParams {
     const PSegment *segs;
@@ -72,6 +83,10 @@ struct PParams {
     int64_t total_tasks;
     unsigned long long *queue;
     int *measured, *tiles_done;
+    unsigned long long *ready;  // [m-tiles of all segments]: (segment + 1) << 32 | m-tile, in order of completion
+    int *ready_tail;            // entries published
+    unsigned long long *measure_queue;  // next 32-row measurement
+    int64_t total_measures;
     int stages, a_planes, b_planes, nprod;
     uint32_t prod_code, stage_bytes;
     uint64_t limit_ns;
@@ -119,6 +134,26 @@ __device__ __forceinline__ bool wait_counter(const int *cnt, int target, const P
     return true;
 }
 
+// As wait_counter, for a published entry of the measurement list (non-zero).
+__device__ __forceinline__ bool wait_entry(const unsigned long long *entry, const PParams &p, unsigned long long *e,
+                                           bool *timed_out) {
+    *timed_out = false;
+    if ((*e = ld_acquire_gpu(entry)) != 0) return true;
+    const uint64_t t0 = global_ns();
+    uint32_t iter = 0;
+    while ((*e = ld_acquire_gpu(entry)) == 0) {
+        __nanosleep(100);
+        if (((++iter) & 31u) == 0u) {
+            if (*reinterpret_cast<volatile int *>(p.err) != 0) return false;
+            if (global_ns() - t0 > p.limit_ns) {
+                *timed_out = true;
+                return false;
+            }
+        }
+    }
+    return true;
+}
+
 __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const PParams p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -130,16 +165,14 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
     uint64_t *drain = tempty + 2;
     uint64_t *task_full = drain + 1;            // [kTaskRing] task published by the producer
     uint64_t *task_empty = task_full + kTaskRing;  // [kTaskRing] read by the MMA thread and the epilogue
-    uint64_t *mfull = task_empty + kTaskRing;    // [kMRing] m-tile handed to the measurement warps
-    uint64_t *mempty = mfull + kMRing;
-    int64_t *task_id = reinterpret_cast<int64_t *>(mempty + kMRing);  // [kTaskRing]
-    int *task_seg = reinterpret_cast<int *>(task_id + kTaskRing);    // [kTaskRing]
-    int *m_seg = task_seg + kTaskRing;                               // [kMRing]
-    int *m_mt = m_seg + kMRing;                                      // [kMRing]
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(m_mt + kMRing);
+    int64_t *task_id = reinterpret_cast<int64_t *>(task_empty + kTaskRing);  // [kTaskRing]
+    int *task_seg = reinterpret_cast<int *>(task_id + kTaskRing);           // [kTaskRing]
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(task_seg + kTaskRing);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    int *m_sstar = reinterpret_cast<int *>(tmem_slot + 4);      // [128]
-    float *m_scale = reinterpret_cast<float *>(m_sstar + kBM);  // [128]
+    int *m_now = reinterpret_cast<int *>(tmem_slot + 4);             // [group][segment or -1, m-tile, part]
+    int *m_sstar = m_now + 4 * kMeasureGroups;                       // [group][32]
+    float *m_scale = reinterpret_cast<float *>(m_sstar + 32 * kMeasureGroups);  // [group][32]
+    double *m_sums = reinterpret_cast<double *>(reinterpret_cast<uint8_t *>(full) + kPBarrierBytes);  // [group][kMeasureSums]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -155,10 +188,6 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
         for (int r = 0; r < kTaskRing; ++r) {
             mbar_init(&task_full[r], 1);
             mbar_init(&task_empty[r], 2);
-        }
-        for (int r = 0; r < kMRing; ++r) {
-            mbar_init(&mfull[r], 1);
-            mbar_init(&mempty[r], kBM);
         }
         *abort_flag = 0;
         fence_mbar_init();
@@ -200,7 +229,7 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
                 const int64_t lt = t - sg->task_begin;
                 const int mt = (int)(lt / sg->num_n_tiles);
                 const int nt = (int)(lt - (int64_t)mt * sg->num_n_tiles);
-                const int target = sg->step + p.stall;
+                const int target = (sg->step + p.stall) * kMeasureParts;
                 if (target > 0) {
                     bool timed_out;
                     if (!wait_counter(p.measured + sg->slot_base + mt, target, p, &timed_out)) {
@@ -309,8 +338,6 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
     } else if (warp < 6) {
         // ---------------- epilogue: warps 2..5 ----------------
         const int quad = warp & 3;
-        int ring = 0;
-        uint32_t ring_phase = 0;
         for (int64_t seq = 0;; ++seq) {
             const int slot = (int)(seq % kTaskRing);
             const bool got = mbar_wait_bounded(&task_full[slot], (uint32_t)((seq / kTaskRing) & 1), abort_flag,
@@ -361,66 +388,74 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
             tc_fence_before();
             mbar_arrive(&tempty[buf]);
             if (valid) sg->P[(int64_t)row * sg->ldP + nt] = ss;
-            // count the tile; the block that finishes the m-tile's last tile measures it
+            // count the tile; the m-tile's last tile puts it on the measurement list
             named_bar_sync(1, 128);
             if (threadIdx.x == 64) {
                 __threadfence();  // the group's stores (ordered by the barrier) before the count
                 const int old = atomicAdd(p.tiles_done + sg->done_base + mt, 1);
                 if (old == sg->num_n_tiles - 1) {
                     __threadfence();  // every block's tiles of this m-tile before the measurement reads them
-                    if (!mbar_wait_bounded(&mempty[ring], ring_phase ^ 1u, abort_flag, p.limit_ns)) {
-                        record_error(p.err, abort_flag, kDevTimeoutEpilogue);
-                    } else {
-                        m_seg[ring] = si;
-                        m_mt[ring] = mt;
-                        mbar_arrive(&mfull[ring]);
-                        if (++ring == kMRing) {
-                            ring = 0;
-                            ring_phase ^= 1u;
-                        }
-                    }
+                    const int at = atomicAdd(p.ready_tail, 1);
+                    st_release_gpu(p.ready + at, (unsigned long long)(si + 1) << 32 | (unsigned)mt);
                 }
             }
             __syncwarp();
         }
-        if (threadIdx.x == 64) {
-            // no more tiles from this block: stop the measurement warps
-            if (mbar_wait_bounded(&mempty[ring], ring_phase ^ 1u, abort_flag, p.limit_ns)) {
-                m_seg[ring] = -1;
-                mbar_arrive(&mfull[ring]);
-            }
-        }
     } else {
-        // ---------------- measurement: warps 6..9 ----------------
-        const int m = threadIdx.x - 192;  // the row of the m-tile this thread draws
-        int ring = 0;
-        uint32_t ring_phase = 0;
+        // ---------------- measurement: warps 6..9 and 10..13, each group on its own ----------------
+        const int g = (warp - 6) >> 2;
+        const int m = threadIdx.x - 192 - 128 * g;  // thread of the group
+        int *now = m_now + 4 * g, *sstar = m_sstar + 32 * g;
+        float *scale = m_scale + 32 * g;
+        double *sums = m_sums + kMeasureSums * g;
         while (true) {
-            const bool ready = mbar_wait_bounded(&mfull[ring], ring_phase, abort_flag, p.limit_ns);
-            if (named_bar_any(2, 128, !ready)) {
-                record_error(p.err, abort_flag, kDevTimeoutMeasure);
-                break;
+            if (m == 0) {
+                int si = -1;
+                const int64_t q = (int64_t)atomicAdd(p.measure_queue, 1ull);
+                if (q < p.total_measures) {
+                    unsigned long long e = 0;
+                    bool timed_out;
+                    if (wait_entry(p.ready + q / kMeasureParts, p, &e, &timed_out)) {
+                        si = (int)(e >> 32) - 1;
+                        now[1] = (int)(unsigned)e;
+                        now[2] = (int)(q % kMeasureParts);
+                    } else if (timed_out) {
+                        record_error(p.err, abort_flag, kDevTimeoutMeasure);
+                    }
+                }
+                now[0] = si;
             }
-            const int si = m_seg[ring];
-            const int mt = m_mt[ring];
-            mbar_arrive(&mempty[ring]);
-            if (++ring == kMRing) {
-                ring = 0;
-                ring_phase ^= 1u;
-            }
+            named_bar_sync(2 + g, 128);
+            const int si = now[0];
             if (si < 0) break;
+            const int mt = now[1];
             const MeasureArgs &a = p.meas[si];
-            const int rows = p.segs[si].rows_valid;
-            const int row = mt * kBM + m;
-            int sstar = 0;
-            float scale = 0.f;
-            if (row < rows) sstar = measure_draw(a, row, &scale);
-            m_sstar[m] = sstar;
-            m_scale[m] = scale;
-            named_bar_sync(2, 128);
-            measure_write_rows(a, m, 128, mt * kBM, min(kBM, rows - mt * kBM), m_sstar, m_scale);
-            named_bar_sync(2, 128);  // the m-tile's next left rows are written
-            if (threadIdx.x == 192) {
+            const int r0 = mt * kBM + now[2] * (kBM / kMeasureParts);
+            const int count = min(kBM / kMeasureParts, p.segs[si].rows_valid - r0);
+            const int d = a.d, T = a.tiles_per_s;
+            const bool in_smem = d * (kBM / kMeasureParts) <= kMeasureSums;
+            if (in_smem) {
+                for (int e = m; e < count * d; e += 128) {
+                    const int r = e / d;
+                    sums[e] = sum_tiles(a.P + (int64_t)(r0 + r) * a.ldP + (e - r * d) * T, T);
+                }
+                named_bar_sync(2 + g, 128);
+            }
+            double Z = 0.0, ws = 0.0;
+            bool ok = false;
+            const RowSums w{in_smem ? sums + m * d : nullptr, a.P + (int64_t)(r0 + m) * a.ldP, d, T};
+            if (m < count) {
+                const int s = draw_row(w, sample_uniform(a.seed, a.n_base + (uint64_t)(r0 + m), a.k, a.job), &Z, &ws, &ok);
+                sstar[m] = s;
+                scale[m] = ok ? rsqrtf((float)ws) : 0.f;
+                a.outcomes[r0 + m] = (uint8_t)s;
+            }
+            named_bar_sync(2 + g, 128);
+            // the logarithm (before the rows are released: the next step adds to the same entry)
+            if (m < count) measure_finish(a, r0 + m, ws, Z, ok, __ldcg(a.logp + a.row0 + r0 + m), w);
+            write_rows_flat<4>(a, m, 128, r0, count, sstar, scale);
+            named_bar_sync(2 + g, 128);  // the next left rows are written
+            if (m == 0) {
                 fence_proxy_async_global();
                 red_release_add_gpu(p.measured + p.segs[si].slot_base + mt, 1);
             }
@@ -454,6 +489,10 @@ cudaError_t launch_batch_persistent(const PersistentArgs &g, int num_sms, int *d
     p.queue = reinterpret_cast<unsigned long long *>(g.queue);
     p.measured = g.measured;
     p.tiles_done = g.tiles_done;
+    p.ready = reinterpret_cast<unsigned long long *>(g.ready);
+    p.ready_tail = g.ready_tail;
+    p.measure_queue = reinterpret_cast<unsigned long long *>(g.measure_queue);
+    p.total_measures = g.total_m_tiles * kMeasureParts;
     p.a_planes = g.a_planes;
     p.b_planes = g.b_planes;
     p.nprod = g.nprod;
@@ -461,13 +500,13 @@ cudaError_t launch_batch_persistent(const PersistentArgs &g, int num_sms, int *d
     for (int q = 0; q < g.nprod; ++q)
         p.prod_code |= ((uint32_t)g.prod_a[q] | ((uint32_t)g.prod_b[q] << 2)) << (4 * q);
     p.stage_bytes = (uint32_t)g.a_planes * kATileBytes + (uint32_t)g.b_planes * kBPlaneBytesMax;
-    p.stages = (kSmemLimit - 1024 - kPBarrierBytes) / (int)p.stage_bytes;
+    p.stages = (kSmemLimit - 1024 - kPBarrierBytes - kPMeasureBytes) / (int)p.stage_bytes;
     if (p.stages > kMaxStages) p.stages = kMaxStages;
     if (p.stages < 2) return cudaErrorInvalidConfiguration;
     p.limit_ns = g.wait_limit_ns;
     p.stall = g.stall_test ? 1 : 0;
     p.err = d_err;
-    const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + kPBarrierBytes;
+    const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + kPBarrierBytes + kPMeasureBytes;
     const int grid = g.total_tasks < num_sms ? (int)g.total_tasks : num_sms;
     tc_batch_persistent_kernel<<<grid, kPThreads, smem, st>>>(p);
     return cudaGetLastError();

@@ -53,3 +53,26 @@ def test_row_groups_give_the_same_bits(precision, chi):
         for n0, N in ((0, 1), (11, 129), (100, 1300), (5, 2600), (1000, 6000)):
             a, l = s.sample(b, 3, N, 4, n0=n0)
             assert np.array_equal(a, smp[n0:n0 + N]) and np.array_equal(l, lp[n0:n0 + N])
+
+
+@pytest.mark.parametrize("precision", ["bf16x2", "bf16x3l"])
+def test_batched_measurements_at_their_edges(precision):
+    """32-row measurements of the batched kernel: row counts around a measurement and an m-tile, chunks of 128
+    rows, and d = 40, whose sums do not fit shared memory.  Bit for bit the jobs sampled alone."""
+    import paper_2512_20064_gb300 as F
+
+    shapes = [(2, 20, 1), (3, 33, 31), (40, 21, 33), (4, 65, 127), (2, 9, 129), (40, 5, 300)]
+    samplers, jobs = [], []
+    for j, (d, chi, N) in enumerate(shapes):
+        b, ts, _ = gen.mps_tensors(7, d, chi, base_seed=60 + j, skew=1.5 if d < 40 else None, dtype=np.complex64)
+        s = F.Sampler(precision=precision)
+        s.load_chain(ts)
+        samplers.append(s)
+        jobs.append(dict(chain=s.h, bonds=b, d=d, N=N, seed=5 + j, job=j, n0=3 * j,
+                         out_samples=np.empty((N, 7), np.uint8), out_logprob=np.empty(N, np.float64)))
+    with F.Sampler(precision=precision, max_microbatch=128) as runner:
+        F.fastmps_sample_batch(runner.h, jobs)
+    for s, j in zip(samplers, jobs):
+        a, l = s.sample(j["bonds"], j["d"], j["N"], j["seed"], n0=j["n0"], job=j["job"])
+        assert np.array_equal(a, j["out_samples"]) and np.array_equal(l, j["out_logprob"])
+        s.close()
