@@ -81,6 +81,7 @@ struct Tensor {
     DevBuf B_hi, B_lo, Bt, B8;
     float fp8_scale = 1.f;  // FP8: stored value = e4m3(A * fp8_scale); FP16: fp16(A * fp8_scale)
     CUtensorMap tmB[2];
+    CUtensorMap tmBh[2];  // boxes of half an n-tile (CTA pairs)
     // streamed operand (pinned host, compact BF16 [chi_l][d][chi_r] (re, im), hi block then lo block)
     DevBuf host_compact;
     int planes = 1;
@@ -148,7 +149,7 @@ bool encode_2d(CUtensorMap *map, CUtensorMapDataType type, int elem_bytes, const
                uint64_t outer, uint64_t ld_elems, uint32_t box_inner, uint32_t box_outer);
 bool encode_2d_bf16(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint64_t ld_elems,
                     uint32_t box_inner, uint32_t box_outer);
-// FP32 contraction scratch [rows][ld] (TMA-store epilogue): 32 x 128 boxes, 128-byte swizzle
+// FP32 contraction scratch [rows][ld] (TMA-store epilogue): boxes of 32 columns x 32 rows, 128-byte swizzle
 bool encode_2d_f32_scratch(CUtensorMap *map, const void *base, uint64_t cols, uint64_t rows, uint64_t ld_elems);
 bool encode_2d_f16(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint64_t ld_elems,
                    uint32_t box_inner, uint32_t box_outer);

@@ -383,17 +383,24 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
                 cudaEventRecord(h->slot_free[cur], st);
                 Bh = h->slot_hi.as<__nv_bfloat16>();
                 Bl = lo;
-                auto map16 = [&](CUtensorMap *m, const void *base) {
-                    return is_f16(h) ? encode_2d_f16(m, base, L.K_pad, L.ncols, L.K_pad, 64, L.bn)
-                                     : encode_2d_bf16(m, base, L.K_pad, L.ncols, L.K_pad, 64, L.bn);
+                auto map16 = [&](CUtensorMap *m, const void *base, int cols) {
+                    return is_f16(h) ? encode_2d_f16(m, base, L.K_pad, L.ncols, L.K_pad, 64, cols)
+                                     : encode_2d_bf16(m, base, L.K_pad, L.ncols, L.K_pad, 64, cols);
                 };
-                if (!map16(&ta.tmB[0], Bh) || (Bl && !map16(&ta.tmB[1], Bl)))
+                if (!map16(&ta.tmB[0], Bh, L.bn) || (Bl && !map16(&ta.tmB[1], Bl, L.bn)) ||
+                    !map16(&ta.tmBh[0], Bh, L.bn / 2) || (Bl && !map16(&ta.tmBh[1], Bl, L.bn / 2)))
                     return fail(h, FASTMPS_ERR_CUDA, "tensor map encoding failed");
-                if (!Bl) ta.tmB[1] = ta.tmB[0];
+                if (!Bl) {
+                    ta.tmB[1] = ta.tmB[0];
+                    ta.tmBh[1] = ta.tmBh[0];
+                }
             } else {
-                ta.tmB[0] = t->tmB[0];
-                ta.tmB[1] = t->tmB[1];
+                for (int q = 0; q < 2; ++q) {
+                    ta.tmB[q] = t->tmB[q];
+                    ta.tmBh[q] = t->tmBh[q];
+                }
             }
+            ta.has_pair = !fp8;
             ta.a_planes = plan.a_planes;
             ta.b_planes = plan.b_planes;
             ta.nprod = plan.nprod;

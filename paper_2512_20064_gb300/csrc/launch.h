@@ -99,10 +99,12 @@ constexpr int kMaxProducts = 4;
 struct TcArgs {
     bool fp8 = false;  // E4M3 operands (one plane each), kind::f8f6f4
     bool f16 = false;  // FP16 (binary16) operands instead of BF16, kind::f16
-    bool has_tmY = false;  // tmY maps the FP32 scratch (ncols x rows, 32 x 128 boxes): TMA-store epilogue
+    bool has_tmY = false;  // tmY maps the FP32 scratch (ncols x rows, 32 x 32 boxes): TMA-store epilogue
     CUtensorMap tmY;
     CUtensorMap tmA[3];
     CUtensorMap tmB[2];
+    bool has_pair = false;  // tmBh maps the site operand like tmB with boxes of L.bn / 2 columns (CTA pairs)
+    CUtensorMap tmBh[2];
     int a_planes, b_planes;
     int nprod;
     int prod_a[kMaxProducts], prod_b[kMaxProducts];

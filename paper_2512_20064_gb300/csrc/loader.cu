@@ -273,9 +273,14 @@ int load_tensor(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const 
         launch_repack_f16(h->staging.p, dtype == FASTMPS_C128, t.L, t.fp8_scale, t.B_hi.as<uint16_t>(),
                           two ? t.B_lo.as<uint16_t>() : nullptr, h->stream);
         if (!encode_2d_f16(&t.tmB[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn) ||
-            (two && !encode_2d_f16(&t.tmB[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn)))
+            (two && !encode_2d_f16(&t.tmB[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn)) ||
+            !encode_2d_f16(&t.tmBh[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn / 2) ||
+            (two && !encode_2d_f16(&t.tmBh[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn / 2)))
             return fail(h, FASTMPS_ERR_CUDA, "tensor map encoding failed");
-        if (!two) t.tmB[1] = t.tmB[0];
+        if (!two) {
+            t.tmB[1] = t.tmB[0];
+            t.tmBh[1] = t.tmBh[0];
+        }
     } else if (is_bf16(h)) {
         if (tune) {
             std::lock_guard<std::mutex> lock(g_tune_mutex);
@@ -305,7 +310,13 @@ int load_tensor(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const 
             return fail(h, FASTMPS_ERR_CUDA, "tensor map encoding failed");
         if (lo && !encode_2d_bf16(&t.tmB[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn))
             return fail(h, FASTMPS_ERR_CUDA, "tensor map encoding failed");
-        if (!lo) t.tmB[1] = t.tmB[0];
+        if (!encode_2d_bf16(&t.tmBh[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn / 2) ||
+            (lo && !encode_2d_bf16(&t.tmBh[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn / 2)))
+            return fail(h, FASTMPS_ERR_CUDA, "tensor map encoding failed");
+        if (!lo) {
+            t.tmB[1] = t.tmB[0];
+            t.tmBh[1] = t.tmBh[0];
+        }
     } else {
         if (!t.Bt.ensure(op_elems * 4)) return fail(h, FASTMPS_ERR_OOM, "site operand allocation failed");
         launch_repack_f32(h->staging.p, dtype == FASTMPS_C128, t.L, t.Bt.as<float>(), h->stream);

@@ -50,6 +50,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "launch.h"
 #include "measure.cuh"
@@ -65,6 +67,7 @@ constexpr int kThreadsFused = 320;           // + 4 measurement warps
 constexpr int kRing = 4;                     // finished m-tiles queued for the measurement warps
 constexpr int kBarrierBytes = 2048;          // mbarriers, ring, measurement staging
 constexpr uint32_t kYStageBytes = 16384;     // one 128 x 32 FP32 chunk of the scratch tile (two buffers)
+constexpr uint32_t kYWarpBytes = 4096;       // a warp's 32 rows of it
 constexpr uint32_t kTmemCols = 512;          // 2 accumulators x 256 columns
 constexpr uint32_t kAccStride = 256;
 constexpr uint32_t kATileBytes = kBM * kBK * 2;  // 16 KB
@@ -126,10 +129,18 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity) 
 // order.  Fused: the block owns m-tiles blockIdx.x, blockIdx.x + gridDim.x, ...
 // and visits all n-tiles of each (i % num_n_tiles == num_n_tiles - 1 ends an
 // m-tile).  Cluster: the cluster owns m-tiles clusterid, clusterid + nclusters,
-// ... and CTA rank r visits n-tiles r*T .. r*T+T-1 of each.  Returns false past
-// the last tile.
-template <int kMode>
+// ... and CTA rank r visits n-tiles r*T .. r*T+T-1 of each.  Pair: the pairs are
+// dealt (two m-tiles, one n-tile) units round-robin, CTA rank r taking the r-th
+// m-tile (which may lie past the last one).  Returns false past the last tile.
+template <int kMode, bool kPair = false>
 __device__ __forceinline__ bool tile_of(const TcParams &p, int i, int &mt, int &nt) {
+    if (kPair) {
+        const int tile = (int)cluster_id_x() + i * (int)cluster_count_x();
+        const int mp = tile / p.num_n_tiles;
+        nt = tile - mp * p.num_n_tiles;
+        mt = 2 * mp + (int)cluster_ctarank();
+        return 2 * mp < p.num_m_tiles;
+    }
     if (kMode == kClusterFused) {
         const int q = i / p.cl_T;
         nt = (int)cluster_ctarank() * p.cl_T + (i - q * p.cl_T);
@@ -335,6 +346,39 @@ __device__ __forceinline__ void cluster_epilogue(const TcParams &p, uint32_t tme
     }
 }
 
+// One arrival on the barrier that frees an accumulator for the MMA issuer (a pair's issuer is in CTA 0).
+template <bool kPair>
+__device__ __forceinline__ void release_accumulator(uint64_t *tempty) {
+    if (kPair) mbar_arrive_cluster(mapa_shared(smem_u32(tempty), 0));
+    else mbar_arrive(tempty);
+}
+
+// ---------------------------------------------------------------------------
+// Scratch stores.  A warp stages the 32 rows x 32 columns it read from tensor memory in a buffer of its own
+// (128-byte rows, the 128-byte swizzle that the tensor map expects) and its first lane stores them with TMA; no
+// other warp is waited for.  With one 128-row store for four warps, two barriers per 32 columns made the
+// epilogue of a 128 x 256 tile 12 thousand cycles long -- longer than its products at K = 512 (8 thousand).
+// two_buffers: the caller alternates between two buffers, so one earlier store may still be reading.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void stage_and_store(const CUtensorMap *tmY, uint8_t *buf, const uint32_t (&r)[32], int lane,
+                                                int x, int y, int rows_valid, bool two_buffers) {
+    if (lane == 0) {
+        if (two_buffers) bulk_wait_read_1();
+        else bulk_wait_read_0();
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        *reinterpret_cast<uint4 *>(buf + lane * 128 + ((j ^ (lane & 7)) * 16)) =
+            make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0 && y < rows_valid) {
+        tma_store_2d(tmY, buf, x, y);
+        bulk_commit();
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Split-K variant: a cluster of S CTAs computes one output tile, CTA rank j
 // accumulating k-blocks [j*nkb/S, (j+1)*nkb/S) in its own tensor memory.  Ranks
@@ -440,7 +484,9 @@ __device__ __forceinline__ void splitk_epilogue(const TcParams &p, const CUtenso
             fence_proxy_async_smem();
             named_bar_sync(1, 128);
             if (threadIdx.x == 64) {
-                tma_store_2d(tmY, sb, nt * p.bn + ch * 32, mt * kBM);
+                for (int q = 0; q < 4; ++q)
+                    if (mt * kBM + 32 * q < p.rows_valid)
+                        tma_store_2d(tmY, sb + q * kYWarpBytes, nt * p.bn + ch * 32, mt * kBM + 32 * q);
                 bulk_commit();
             }
         }
@@ -460,21 +506,21 @@ __device__ __forceinline__ void splitk_epilogue(const TcParams &p, const CUtenso
 // tensor cores' accumulation then spans a few k-blocks only, where its partial
 // sums are small, and the long sum over the whole index is taken with correctly
 // rounded FP32 additions.  The tile is stored like the two-pass epilogue (TMA
-// stores of 128 x 32 chunks, each half through its own staging buffer) and
+// stores of 32 x 32 chunks, each warp through its own staging buffer) and
 // the row's sum of squares is the sum of the two halves' sums.
 // ---------------------------------------------------------------------------
+template <bool kPair>
 __device__ __forceinline__ void promoted_epilogue(const TcParams &p, const CUtensorMap *tmY, uint32_t tmem_base,
                                                   uint64_t *tfull, uint64_t *tempty, uint8_t *ystage, float *ss_hi,
                                                   volatile int *abort_flag, int warp, int lane) {
     const int quad = warp & 3;
     const int half = (warp - 4) >> 2;        // 0: columns 0..127 of the tile, 1: columns 128..255
     const int rl = quad * 32 + lane;
-    const int elected = half == 0 ? 128 : 256;  // first thread of each half
     const int nch = (p.num_k_blocks + p.kchunk - 1) / p.kchunk;
-    uint8_t *sb = ystage + (uint32_t)half * kYStageBytes;  // this half's staging buffer
+    uint8_t *sb = ystage + (uint32_t)(half * 4 + quad) * kYWarpBytes;  // this warp's staging buffer
     uint32_t cq = 0;  // chunks consumed (buffer cq % 2)
     int mt, nt;
-    for (int i = 0; tile_of<kPromoted>(p, i, mt, nt); ++i) {
+    for (int i = 0; tile_of<kPromoted, kPair>(p, i, mt, nt); ++i) {
         float acc[128];
         for (int c = 0; c < nch; ++c, ++cq) {
             const int buf = (int)(cq & 1u);
@@ -511,7 +557,7 @@ __device__ __forceinline__ void promoted_epilogue(const TcParams &p, const CUten
             // the warp's tensor-memory reads are complete: one arrive per warp frees the buffer
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[buf]);
+            if (lane == 0) release_accumulator<kPair>(&tempty[buf]);
         }
         const int row = mt * kBM + rl;
         float ss = 0.f;
@@ -519,19 +565,10 @@ __device__ __forceinline__ void promoted_epilogue(const TcParams &p, const CUten
         for (int g = 0; g < 4; ++g) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) ss = fmaf(acc[g * 32 + j], acc[g * 32 + j], ss);
-            if (threadIdx.x == elected) bulk_wait_read_0();  // this half's previous store has read sb
-            named_bar_sync(2 + half, 128);
+            uint32_t r[32];
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                *reinterpret_cast<float4 *>(sb + rl * 128 + ((j ^ (rl & 7)) * 16)) =
-                    make_float4(acc[g * 32 + 4 * j], acc[g * 32 + 4 * j + 1], acc[g * 32 + 4 * j + 2],
-                                acc[g * 32 + 4 * j + 3]);
-            fence_proxy_async_smem();
-            named_bar_sync(2 + half, 128);
-            if (threadIdx.x == elected) {
-                tma_store_2d(tmY, sb, nt * p.bn + half * 128 + g * 32, mt * kBM);
-                bulk_commit();
-            }
+            for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(acc[g * 32 + j]);
+            stage_and_store(tmY, sb, r, lane, nt * p.bn + half * 128 + g * 32, mt * kBM + quad * 32, p.rows_valid, false);
         }
         // the row's sum of squares: low half + high half
         if (half == 1) ss_hi[rl] = ss;
@@ -539,10 +576,10 @@ __device__ __forceinline__ void promoted_epilogue(const TcParams &p, const CUten
         if (half == 0 && row < p.rows_valid) p.P[(int64_t)row * p.ldP + nt] = ss + ss_hi[rl];
         named_bar_sync(1, 256);  // ss_hi is free for the next tile
     }
-    if (threadIdx.x == elected) bulk_wait_all();
+    if (lane == 0) bulk_wait_all();
 }
 
-template <int kMode, bool kFp8>
+template <int kMode, bool kFp8, bool kPair = false>
 __global__ void __launch_bounds__(kMode == kFusedCta ? kThreadsFused : (kMode == kPromoted ? kThreadsPromoted : kThreads), 1)
 tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmA1,
                    const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB0,
@@ -552,6 +589,8 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
     constexpr bool kCluster = kMode == kClusterFused;
     constexpr bool kSplit = kMode == kSplitK;
     constexpr bool kPromo = kMode == kPromoted;
+    static_assert(!kPair || ((kMode == kTwoPass || kMode == kPromoted) && !kFp8), "no such pair variant");
+    const uint32_t pair_rank = kPair ? cluster_ctarank() : 0u;
     // split-K: this CTA's share of the k-blocks
     const int kb_lo = kSplit ? (int)(cluster_ctarank() * (uint32_t)p.num_k_blocks / (uint32_t)p.ksplit) : 0;
     const int kb_hi = kSplit ? (int)((cluster_ctarank() + 1) * (uint32_t)p.num_k_blocks / (uint32_t)p.ksplit)
@@ -587,7 +626,8 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
         }
         for (int b = 0; b < 4; ++b) {
             mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], kPromo ? 8 : 128);  // promoted: one arrive per epilogue warp
+            // one arrive per epilogue warp (promoted, pair: of both CTAs), else per epilogue thread
+            mbar_init(&tempty[b], kPair ? (kPromo ? 16 : 8) : kPromo ? 8 : 128);
         }
         mbar_init(drain, 1);
         for (int r = 0; r < kRing; ++r) {
@@ -618,13 +658,17 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
         if (p.b_planes > 1) prefetch_tmap(&tmB1);
     }
     if (warp == 1) {
-        tmem_alloc(tmem_slot, kTmemCols);
-        tmem_relinquish();
+        if (kPair) {
+            tmem_alloc_pair(tmem_slot, kTmemCols);
+        } else {
+            tmem_alloc(tmem_slot, kTmemCols);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
     __syncthreads();
     // cluster variants: every CTA's barriers are initialised before any remote arrive
-    if (kCluster || kSplit) cluster_sync_all();
+    if (kCluster || kSplit || kPair) cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     // ---------------- TMA producer (warp 0) ----------------
@@ -636,9 +680,9 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
             for (int s = 0; s < kMaxStages; ++s) last_parity[s] = -1;
             bool failed = false;
             int mt, nt;
-            for (int i = 0; !failed && tile_of<kMode>(p, i, mt, nt); ++i) {
+            for (int i = 0; !failed && tile_of<kMode, kPair>(p, i, mt, nt); ++i) {
                 const int y_a = p.row0 + mt * kBM;
-                const int y_b = nt * p.bn;
+                const int y_b = nt * p.bn + (int)pair_rank * (p.bn / 2);  // pair: this CTA's half of the tile's columns
                 for (int kb = kb_lo; kb < kb_hi; ++kb) {
                     if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, abort_flag)) {
                         record_error(p.err, abort_flag, kDevTimeoutProducer);
@@ -646,14 +690,25 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
                         break;
                     }
                     uint8_t *sbase = smem + (size_t)stage * p.stage_bytes;
-                    mbar_arrive_expect_tx(&full[stage], p.stage_bytes);
                     const int x = kb * (kFp8 ? 2 * kBK : kBK);  // 128-byte rows: 64 BF16 or 128 FP8
-                    tma_load_2d(sbase, &tmA0, &full[stage], x, y_a);
-                    if (p.a_planes > 1) tma_load_2d(sbase + kATileBytes, &tmA1, &full[stage], x, y_a);
-                    if (p.a_planes > 2) tma_load_2d(sbase + 2 * kATileBytes, &tmA2, &full[stage], x, y_a);
                     uint8_t *bbase = sbase + (size_t)p.a_planes * kATileBytes;
-                    tma_load_2d(bbase, &tmB0, &full[stage], x, y_b);
-                    if (p.b_planes > 1) tma_load_2d(bbase + p.b_plane_bytes, &tmB1, &full[stage], x, y_b);
+                    if (kPair) {
+                        // both CTAs' copies complete on the leader's barrier, which expects them all
+                        const uint32_t bar = mapa_shared(smem_u32(&full[stage]), 0);
+                        if (pair_rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * p.stage_bytes);
+                        tma_load_2d_pair(sbase, &tmA0, bar, x, y_a);
+                        if (p.a_planes > 1) tma_load_2d_pair(sbase + kATileBytes, &tmA1, bar, x, y_a);
+                        if (p.a_planes > 2) tma_load_2d_pair(sbase + 2 * kATileBytes, &tmA2, bar, x, y_a);
+                        tma_load_2d_pair(bbase, &tmB0, bar, x, y_b);
+                        if (p.b_planes > 1) tma_load_2d_pair(bbase + p.b_plane_bytes, &tmB1, bar, x, y_b);
+                    } else {
+                        mbar_arrive_expect_tx(&full[stage], p.stage_bytes);
+                        tma_load_2d(sbase, &tmA0, &full[stage], x, y_a);
+                        if (p.a_planes > 1) tma_load_2d(sbase + kATileBytes, &tmA1, &full[stage], x, y_a);
+                        if (p.a_planes > 2) tma_load_2d(sbase + 2 * kATileBytes, &tmA2, &full[stage], x, y_a);
+                        tma_load_2d(bbase, &tmB0, &full[stage], x, y_b);
+                        if (p.b_planes > 1) tma_load_2d(bbase + p.b_plane_bytes, &tmB1, &full[stage], x, y_b);
+                    }
                     last_parity[stage] = (int)phase;
                     if (++stage == p.stages) {
                         stage = 0;
@@ -663,15 +718,30 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
             }
             if (failed) {
                 // let the copies this thread issued land before shared memory is released
-                for (int s = 0; s < p.stages; ++s)
-                    if (last_parity[s] >= 0) mbar_wait_drain(&full[s], (uint32_t)last_parity[s]);
+                if (kPair && pair_rank != 0) {
+                    // no barrier of this CTA counts them: they land long before this
+                    const uint64_t t0 = global_ns();
+                    while (global_ns() - t0 < 10000000ull) {
+                    }
+                } else {
+                    for (int s = 0; s < p.stages; ++s)
+                        if (last_parity[s] >= 0) mbar_wait_drain(&full[s], (uint32_t)last_parity[s]);
+                }
             }
         }
         __syncwarp();
     };
-    // ---------------- MMA issuer (warp 1) ----------------
+    // ---------------- MMA issuer (warp 1; of a pair, the leader's) ----------------
     auto run_mma = [&]() {
-        if (lane == 0) {
+        auto accumulator_free = [&](int b, uint32_t parity) {
+            return kPair ? mbar_wait_cluster_bounded(&tempty[b], parity, abort_flag)
+                         : mbar_wait_bounded(&tempty[b], parity, abort_flag);
+        };
+        auto commit = [&](uint64_t *bar) {
+            if (kPair) tc_commit_pair(bar);
+            else tc_commit(bar);
+        };
+        if (lane == 0 && pair_rank == 0) {
             int stage = 0;
             uint32_t phase = 0;
             int lt = 0;
@@ -679,12 +749,12 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
             bool issued = false;
             int mt, nt;
             uint32_t cq = 0;  // promoted accumulation: chunks issued so far (buffer cq % 2)
-            for (int i = 0; !failed && tile_of<kMode>(p, i, mt, nt); ++i, ++lt) {
+            for (int i = 0; !failed && tile_of<kMode, kPair>(p, i, mt, nt); ++i, ++lt) {
                 int buf = lt & 1;
                 uint32_t d_tmem = 0;
                 if (!kPromo) {
                     const uint32_t use = (uint32_t)(lt >> 1);
-                    if (!mbar_wait_bounded(&tempty[buf], (use & 1u) ^ 1u, abort_flag)) {
+                    if (!accumulator_free(buf, (use & 1u) ^ 1u)) {
                         record_error(p.err, abort_flag, kDevTimeoutMma);
                         failed = true;
                         break;
@@ -698,7 +768,7 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
                         // a fresh 128-column accumulator for the next chunk of the contraction index
                         buf = (int)(cq & 1u);
                         const uint32_t use = cq >> 1;
-                        if (!mbar_wait_bounded(&tempty[buf], (use & 1u) ^ 1u, abort_flag)) {
+                        if (!accumulator_free(buf, (use & 1u) ^ 1u)) {
                             record_error(p.err, abort_flag, kDevTimeoutMma);
                             failed = true;
                             break;
@@ -726,29 +796,31 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
                             // +32 bytes along K inside the swizzle row = +2 in the address field
                             // (16 BF16 or 32 FP8 elements per MMA)
                             const uint32_t acc = (kin | q | k16) != 0 ? 1u : 0u;
-                            if (kFp8)
+                            if (kPair)
+                                tc_mma_bf16_pair(d_tmem, ad + (uint64_t)(2 * k16), bd + (uint64_t)(2 * k16), p.idesc, acc);
+                            else if (kFp8)
                                 tc_mma_f8(d_tmem, ad + (uint64_t)(2 * k16), bd + (uint64_t)(2 * k16), p.idesc, acc);
                             else
                                 tc_mma_bf16(d_tmem, ad + (uint64_t)(2 * k16), bd + (uint64_t)(2 * k16), p.idesc, acc);
                         }
                     }
                     issued = true;
-                    tc_commit(&empty[stage]);
+                    commit(&empty[stage]);
                     if (++stage == p.stages) {
                         stage = 0;
                         phase ^= 1u;
                     }
                     if (kPromo && (kin == p.kchunk - 1 || kb == kb_hi - 1)) {
-                        tc_commit(&tfull[buf]);
+                        commit(&tfull[buf]);
                         ++cq;
                     }
                 }
                 if (failed) break;
-                if (!kPromo) tc_commit(&tfull[buf]);
+                if (!kPromo) commit(&tfull[buf]);
             }
             if (failed && issued) {
                 // wait for this thread's outstanding MMAs before tensor memory is freed
-                tc_commit(drain);
+                commit(drain);
                 mbar_wait_drain(drain, 0u);
             }
         }
@@ -766,7 +838,7 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
         } else {
             setmaxnreg_inc<kPromoRegsEpi>();
             // ---------------- promoted-accumulation epilogue: warps 4..11 ----------------
-            promoted_epilogue(p, &tmY, tmem_base, tfull, tempty, ystage, m_scale, abort_flag, warp, lane);
+            promoted_epilogue<kPair>(p, &tmY, tmem_base, tfull, tempty, ystage, m_scale, abort_flag, warp, lane);
         }
     } else if (warp == 0) {
         run_producer();
@@ -785,13 +857,13 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
         int ring = 0;               // (fused) next ring slot and its phase, tracked by thread 64
         uint32_t ring_phase = 0;
         int mt, nt;
-        int chunk = 0;  // chunks staged so far (alternating staging buffers)
-        const bool group_sync = kFused || p.tma_store;
-        for (int i = 0; tile_of<kMode>(p, i, mt, nt); ++i, ++lt) {
+        uint32_t chunk = 0;  // chunks this warp has staged (two 4 KB buffers in turn)
+        for (int i = 0; tile_of<kMode, kPair>(p, i, mt, nt); ++i, ++lt) {
             const int buf = lt & 1;
             const uint32_t use = (uint32_t)(lt >> 1);
             const bool ready = mbar_wait_bounded(&tfull[buf], use & 1u, abort_flag);
-            if (group_sync ? named_bar_any(1, 128, !ready) : !ready) {
+            // the fused variant's warps decide together (they meet at a barrier below), the others on their own
+            if (kFused ? named_bar_any(1, 128, !ready) : !__all_sync(0xffffffffu, ready)) {
                 record_error(p.err, abort_flag, kDevTimeoutEpilogue);
                 break;
             }
@@ -801,33 +873,16 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
             float *yrow = p.Y + (int64_t)row * p.ldY + (int64_t)nt * p.bn;
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)buf * kAccStride;
             float ss = 0.f;
-            for (int ch = 0; ch < p.bn / 32; ++ch) {
-                uint32_t r[32];
-                tmem_ld_32x32b_x32(taddr + (uint32_t)(ch * 32), r);
-                tc_wait_ld();
+            const int nch = p.bn / 32;
+            auto put_chunk = [&](const uint32_t (&r)[32], int ch) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
                     const float v = __uint_as_float(r[j]);
                     ss = fmaf(v, v, ss);
                 }
                 if (!kFused && p.tma_store) {
-                    // stage the 128 x 32 chunk (row = TMEM lane) with the 128-byte swizzle the tensor
-                    // map expects, then one thread stores it with TMA
-                    uint8_t *sb = ystage + (uint32_t)(chunk & 1) * kYStageBytes;
-                    if (threadIdx.x == 64) bulk_wait_read_1();  // the store two chunks back has read sb
-                    named_bar_sync(1, 128);
-                    const int rl = quad * 32 + lane;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        *reinterpret_cast<float4 *>(sb + rl * 128 + ((j ^ (rl & 7)) * 16)) =
-                            make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                        __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
-                    fence_proxy_async_smem();
-                    named_bar_sync(1, 128);
-                    if (threadIdx.x == 64) {
-                        tma_store_2d(&tmY, sb, nt * p.bn + ch * 32, mt * kBM);
-                        bulk_commit();
-                    }
+                    stage_and_store(&tmY, ystage + (uint32_t)(quad * 2) * kYWarpBytes + (chunk & 1u) * kYWarpBytes, r,
+                                    lane, nt * p.bn + ch * 32, mt * kBM + quad * 32, p.rows_valid, true);
                     ++chunk;
                 } else if (valid) {
                     float4 *dst = reinterpret_cast<float4 *>(yrow + ch * 32);
@@ -836,9 +891,28 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
                         dst[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
                                              __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
                 }
+            };
+            // the next 32 columns are on their way from tensor memory while a chunk is squared and staged
+            uint32_t ra[32], rb[32];
+            tmem_ld_32x32b_x32(taddr, ra);
+            tc_wait_ld_for(ra);
+            for (int ch = 0; ch < nch; ch += 2) {
+                const bool two = ch + 1 < nch, more = ch + 2 < nch;
+                if (two) tmem_ld_32x32b_x32(taddr + (uint32_t)((ch + 1) * 32), rb);
+                put_chunk(ra, ch);
+                if (!two) break;
+                tc_wait_ld_for(rb);
+                if (more) tmem_ld_32x32b_x32(taddr + (uint32_t)((ch + 2) * 32), ra);
+                put_chunk(rb, ch + 1);
+                if (more) tc_wait_ld_for(ra);
             }
             tc_fence_before();
-            mbar_arrive(&tempty[buf]);
+            if (kPair) {
+                __syncwarp();
+                if (lane == 0) release_accumulator<true>(&tempty[buf]);
+            } else {
+                mbar_arrive(&tempty[buf]);
+            }
             if (valid) p.P[(int64_t)row * p.ldP + nt] = ss;
             if (kFused && (i + 1) % p.num_n_tiles == 0) {
                 // the m-tile is complete: the group barrier orders the 128 threads' stores before
@@ -859,7 +933,7 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
                 __syncwarp();
             }
         }
-        if (!kFused && p.tma_store && threadIdx.x == 64) bulk_wait_all();  // scratch stores complete
+        if (!kFused && p.tma_store && lane == 0) bulk_wait_all();  // this warp's scratch stores are complete
         if (kFused && threadIdx.x == 64) {
             // no more m-tiles from this block: stop the measurement warps
             if (mbar_wait_bounded(&mempty[ring], ring_phase ^ 1u, abort_flag)) {
@@ -900,11 +974,40 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
     tc_fence_before();
     __syncthreads();
     // cluster variants: no CTA leaves while another may still read its shared memory or arrive on its barriers
-    if (kCluster || kSplit) cluster_sync_all();
+    if (kCluster || kSplit || kPair) cluster_sync_all();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, kTmemCols);
+        if (kPair) tmem_dealloc_pair(tmem_base, kTmemCols);
+        else tmem_dealloc(tmem_base, kTmemCols);
     }
+}
+
+// Whether a launch runs on CTA pairs (see kPair): if its units of two m-tiles and one n-tile, one per pair, take no
+// more rounds than its tiles, one per CTA -- an odd last m-tile leaves half a pair idle.
+bool pair_pays(const TcArgs &a, const TcParams &p, int num_sms) {
+    if (!a.has_pair || a.fp8 || p.bn < 128 || p.num_m_tiles < 2) return false;
+    const int64_t pairs = num_sms / 2, units = (int64_t)((p.num_m_tiles + 1) / 2) * p.num_n_tiles;
+    const int64_t tiles = (int64_t)p.num_m_tiles * p.num_n_tiles;
+    return (units + pairs - 1) / pairs <= (tiles + num_sms - 1) / num_sms;
+}
+
+template <class Kernel>
+cudaError_t launch_pairs(Kernel kern, int units, int num_sms, int threads, size_t smem, cudaStream_t st, const TcArgs &a,
+                         const TcParams &p) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(2 * std::min(units, num_sms / 2)));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const CUtensorMap &a1 = a.tmA[a.a_planes > 1 ? 1 : 0], &a2 = a.tmA[a.a_planes > 2 ? 2 : 0];
+    return cudaLaunchKernelEx(&cfg, kern, a.tmA[0], a1, a2, a.tmBh[0], a.tmBh[a.b_planes > 1 ? 1 : 0], a.tmY, p);
 }
 
 int stages_for(uint32_t stage_bytes, uint32_t extra = 0) {
@@ -945,6 +1048,11 @@ cudaError_t launch_contract_tc(const TcArgs &a, const SiteLayout &L, const Contr
     p.stage_bytes = (uint32_t)a.a_planes * kATileBytes + (uint32_t)a.b_planes * p.b_plane_bytes;
     p.stages = stages_for(p.stage_bytes);
     if (p.stages < 2) return cudaErrorInvalidConfiguration;
+    const bool pair = !fused && a.has_tmY && pair_pays(a, p, num_sms);
+    if (pair) {
+        p.b_plane_bytes /= 2;  // each CTA holds half of the n-tile's columns
+        p.stage_bytes = (uint32_t)a.a_planes * kATileBytes + (uint32_t)a.b_planes * p.b_plane_bytes;
+    }
     // TMA-store epilogue when the staging buffers fit beside at least two pipeline stages
     p.tma_store = 0;
     if (a.has_tmY && !fused) {
@@ -955,7 +1063,8 @@ cudaError_t launch_contract_tc(const TcArgs &a, const SiteLayout &L, const Contr
         }
     }
     p.row0 = (int)a.row0;
-    p.idesc = a.fp8 ? idesc_e4m3_f32(kBM, L.bn) : (a.f16 ? idesc_f16_f32(kBM, L.bn) : idesc_bf16_f32(kBM, L.bn));
+    const int mma_m = pair ? 2 * kBM : kBM;
+    p.idesc = a.fp8 ? idesc_e4m3_f32(kBM, L.bn) : (a.f16 ? idesc_f16_f32(mma_m, L.bn) : idesc_bf16_f32(mma_m, L.bn));
     if (a.fp8 && (fused || a.a_planes > 2 || a.b_planes != 1)) return cudaErrorInvalidValue;
     p.Y = o.Y;
     p.ldY = o.ldY;
@@ -979,7 +1088,14 @@ cudaError_t launch_contract_tc(const TcArgs &a, const SiteLayout &L, const Contr
     const CUtensorMap &b1 = a.tmB[a.b_planes > 1 ? 1 : 0];
     const CUtensorMap &ty = a.has_tmY ? a.tmY : a.tmA[0];  // unused when p.tma_store == 0
     cudaError_t e;
-    if (a.fp8) {
+    if (pair) {
+        auto kern = tc_contract_kernel<kTwoPass, false, true>;
+        if (!p.tma_store) return cudaErrorInvalidConfiguration;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+        if (e != cudaSuccess) return e;
+        e = launch_pairs(kern, (p.num_m_tiles + 1) / 2 * p.num_n_tiles, num_sms, kThreads, smem, st, a, p);
+        if (e != cudaSuccess) return e;
+    } else if (a.fp8) {
         e = cudaFuncSetAttribute(tc_contract_kernel<kTwoPass, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kSmemLimit);
         if (e != cudaSuccess) return e;
@@ -1218,13 +1334,15 @@ cudaError_t launch_contract_tc_promoted(const TcArgs &a, const SiteLayout &L, co
             return cudaErrorInvalidValue;
         p.prod_code |= ((uint32_t)a.prod_a[q] | ((uint32_t)a.prod_b[q] << 2)) << (4 * q);
     }
-    p.b_plane_bytes = (uint32_t)L.bn * 128;
+    const bool pair = pair_pays(a, p, num_sms);
+    p.b_plane_bytes = (uint32_t)L.bn * (pair ? 64 : 128);  // a CTA of a pair holds half of the n-tile's columns
     p.stage_bytes = (uint32_t)a.a_planes * kATileBytes + (uint32_t)a.b_planes * p.b_plane_bytes;
     p.stages = stages_for(p.stage_bytes, 2 * kYStageBytes);
     if (p.stages < 2) return cudaErrorInvalidConfiguration;
     p.tma_store = 1;
     p.row0 = (int)a.row0;
-    p.idesc = a.f16 ? idesc_f16_f32(kBM, L.bn) : idesc_bf16_f32(kBM, L.bn);
+    const int mma_m = pair ? 2 * kBM : kBM;
+    p.idesc = a.f16 ? idesc_f16_f32(mma_m, L.bn) : idesc_bf16_f32(mma_m, L.bn);
     p.Y = o.Y;
     p.ldY = o.ldY;
     p.P = o.P;
@@ -1238,12 +1356,13 @@ cudaError_t launch_contract_tc_promoted(const TcArgs &a, const SiteLayout &L, co
     const int tiles = p.num_m_tiles * p.num_n_tiles;
     if (tiles <= 0) return cudaSuccess;
     const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + kBarrierBytes + 2 * kYStageBytes;
-    auto kern = tc_contract_kernel<kPromoted, false>;
+    auto kern = pair ? tc_contract_kernel<kPromoted, false, true> : tc_contract_kernel<kPromoted, false, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     // the epilogue warpgroups' register increase is served from the launch's own registers: refuse a
     // build whose launch count would leave the increase waiting
-    static int regs = -1;
+    static int regs_of[2] = {-1, -1};
+    int &regs = regs_of[pair];
     if (regs < 0) {
         cudaFuncAttributes fa;
         e = cudaFuncGetAttributes(&fa, kern);
@@ -1251,6 +1370,10 @@ cudaError_t launch_contract_tc_promoted(const TcArgs &a, const SiteLayout &L, co
         regs = fa.numRegs;
     }
     if (regs * kThreadsPromoted < kPromoRegsCtl * 128 + kPromoRegsEpi * 256) return cudaErrorInvalidConfiguration;
+    if (pair) {
+        e = launch_pairs(kern, (p.num_m_tiles + 1) / 2 * p.num_n_tiles, num_sms, kThreadsPromoted, smem, st, a, p);
+        return e != cudaSuccess ? e : cudaGetLastError();
+    }
     const int grid = tiles < num_sms ? tiles : num_sms;
     const CUtensorMap &a1 = a.tmA[a.a_planes > 1 ? 1 : 0], &a2 = a.tmA[a.a_planes > 2 ? 2 : 0];
     const CUtensorMap &b1 = a.tmB[a.b_planes > 1 ? 1 : 0];
