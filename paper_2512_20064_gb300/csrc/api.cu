@@ -9,6 +9,12 @@ using namespace fastmps;
 
 namespace {
 std::string g_create_error;
+
+// The tensor loaded in slot k, or nullptr.
+Tensor *loaded(const std::map<int, std::unique_ptr<Tensor>> &slots, int k) {
+    auto it = slots.find(k);
+    return it == slots.end() ? nullptr : it->second.get();
+}
 }  // namespace
 
 extern "C" {
@@ -136,7 +142,7 @@ int fastmps_load_site(fastmps_handle h, int k, int chi_l, int d, int chi_r, cons
     cudaSetDevice(h->device);
     std::unique_ptr<Tensor> t(new (std::nothrow) Tensor());
     if (!t) return fail(h, FASTMPS_ERR_OOM, "out of host memory");
-    int rc = load_tensor(h, *t, chi_l, d, chi_r, A, dtype);
+    int rc = load_tensor(h, *t, chi_l, d, chi_r, A, dtype, nullptr, loaded(h->site_tensor, k));
     if (rc) return rc;
     h->site_tensor[k] = std::move(t);
     h->site_pool.erase(k);
@@ -149,7 +155,7 @@ int fastmps_load_pool(fastmps_handle h, int j, int chi_l, int d, int chi_r, cons
     cudaSetDevice(h->device);
     std::unique_ptr<Tensor> t(new (std::nothrow) Tensor());
     if (!t) return fail(h, FASTMPS_ERR_OOM, "out of host memory");
-    int rc = load_tensor(h, *t, chi_l, d, chi_r, A, dtype);
+    int rc = load_tensor(h, *t, chi_l, d, chi_r, A, dtype, nullptr, loaded(h->pool_tensor, j));
     if (rc) return rc;
     h->pool_tensor[j] = std::move(t);
     return FASTMPS_OK;
@@ -209,7 +215,7 @@ int fastmps_load_site_vidal(fastmps_handle h, int k, int chi_l, int d, int chi_r
     cudaSetDevice(h->device);
     std::unique_ptr<Tensor> t(new (std::nothrow) Tensor());
     if (!t) return fail(h, FASTMPS_ERR_OOM, "out of host memory");
-    int rc = load_tensor(h, *t, chi_l, d, chi_r, Gamma, dtype, Lambda);
+    int rc = load_tensor(h, *t, chi_l, d, chi_r, Gamma, dtype, Lambda, loaded(h->site_tensor, k));
     if (rc) return rc;
     h->site_tensor[k] = std::move(t);
     h->site_pool.erase(k);
@@ -224,7 +230,7 @@ int fastmps_load_pool_vidal(fastmps_handle h, int j, int chi_l, int d, int chi_r
     cudaSetDevice(h->device);
     std::unique_ptr<Tensor> t(new (std::nothrow) Tensor());
     if (!t) return fail(h, FASTMPS_ERR_OOM, "out of host memory");
-    int rc = load_tensor(h, *t, chi_l, d, chi_r, Gamma, dtype, Lambda);
+    int rc = load_tensor(h, *t, chi_l, d, chi_r, Gamma, dtype, Lambda, loaded(h->pool_tensor, j));
     if (rc) return rc;
     h->pool_tensor[j] = std::move(t);
     return FASTMPS_OK;

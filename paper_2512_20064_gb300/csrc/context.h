@@ -79,7 +79,7 @@ struct Tensor {
     int measure_mode = 0;  // autotuned: 2 = single-pass cluster kernel for this site, 0 = two-pass
     // resident operands (device)
     DevBuf B_hi, B_lo, Bt, B8;
-    float fp8_scale = 1.f;  // FP8: stored value = e4m3(A * fp8_scale); FP16: fp16(A * fp8_scale)
+    float fp8_scale = 1.f;  // FP8: stored value = e4m3(A * fp8_scale); host-streamed FP16: fp16(A * fp8_scale)
     CUtensorMap tmB[2];
     CUtensorMap tmBh[2];  // boxes of half an n-tile (CTA pairs)
     // streamed operand (pinned host, compact BF16 [chi_l][d][chi_r] (re, im), hi block then lo block)
@@ -213,8 +213,11 @@ bool is_device_ptr(const void *p);
 // ---- loader.cu ----
 // Copy and repack one tensor into t.  lam (nullable, host or device, chi_r entries of the
 // tensor's real type): Vidal form, the stored tensor is A[a][s][b] * lam[b].
+// replaced (nullable): the tensor that t takes the place of; once the arguments have been checked, t may take over its
+// device operands where they fit and are at most twice as large, so that reloading a chain neither frees nor
+// allocates (a free waits for the device).
 int load_tensor(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const void *A, int dtype,
-                const void *lam = nullptr);
+                const void *lam = nullptr, Tensor *replaced = nullptr);
 // The tensor site k uses (its own or its pool entry), or nullptr.
 Tensor *site_tensor_of(fastmps_handle h, int k);
 

@@ -377,8 +377,7 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
                 }
                 cudaStreamWaitEvent(st, h->copy_done[cur], 0);
                 __nv_bfloat16 *lo = plan.b_planes > 1 ? h->slot_lo.as<__nv_bfloat16>() : nullptr;
-                launch_expand_bf16(h->slot_compact[cur].as<__nv_bfloat16>(), t->planes, L,
-                                   h->slot_hi.as<__nv_bfloat16>(), lo, st);
+                launch_expand_bf16(h->slot_compact[cur].as<__nv_bfloat16>(), L, h->slot_hi.as<__nv_bfloat16>(), lo, st);
                 h->stats.launches += 1;
                 cudaEventRecord(h->slot_free[cur], st);
                 Bh = h->slot_hi.as<__nv_bfloat16>();

@@ -67,45 +67,130 @@ __device__ __forceinline__ StackedPos stacked_pos(int c, int kappa, int chi_l, i
     return q;
 }
 
-__global__ void repack_bf16_kernel(const void *__restrict__ src, int is_f64, int chi_l, int d, int chi_r, int Cs,
-                                   int ncols, int K_pad, __nv_bfloat16 *__restrict__ B_hi,
-                                   __nv_bfloat16 *__restrict__ B_lo) {
-    const int64_t total = (int64_t)ncols * K_pad;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i / K_pad);
-        const int kappa = (int)(i - (int64_t)c * K_pad);
-        const StackedPos q = stacked_pos(c, kappa, chi_l, d, chi_r, Cs);
-        float x = 0.f;
-        if (!q.zero) x = q.sign * load_part(src, is_f64, q.cidx, q.re_part ? 0 : 1);
-        __nv_bfloat16 hi, lo;
-        split_bf16(x, hi, lo);
-        B_hi[i] = hi;
-        if (B_lo) B_lo[i] = lo;
+// 16-bit operands (BF16, or FP16 at a power-of-two scale) from complex float or double, optionally with column b
+// scaled by lam[b] (Vidal form, in the input's type), or from a compact 16-bit copy.  Bound by HBM: each complex
+// entry is read once and written four times (twice per plane and outcome column).
+// The operand is the transpose of the tensor's rows: a block reads 64 x 32 entries (a, b) of one outcome along b,
+// keeps them as 16-bit values in shared memory, and writes the four runs of 64 entries along kappa that they make
+// (16-byte stores where chi_l is a multiple of 8).  Reading one entry per stored value along kappa instead, a
+// chi_r-strided gather, took 185 us for chi = 2000, d = 3.
+struct Repack16 {
+    const void *src;       // [chi_l][d][chi_r] complex
+    const void *lam;       // [chi_r] real, or null
+    const float *amax;     // FP16: largest |Re|, |Im| (the scale puts it in [16384, 32768]); null: no scale
+    int chi_l, d, chi_r, Cs, K_pad;
+    int f16;
+    uint16_t *hi, *lo;     // lo: null for one plane
+};
+enum Repack16Source : int { kFromFloat = 0, kFromDouble = 1, kFrom16 = 2 };
+constexpr int kRepackA = 64, kRepackB = 32, kRepackLd = kRepackA + 8;
+
+// Entry e of column b as FP32 (aligned to a whole entry).
+template <int kSource>
+__device__ __forceinline__ float2 repack_value(const Repack16 &r, int64_t e, int b) {
+    if constexpr (kSource == kFromDouble) {
+        double2 x = static_cast<const double2 *>(r.src)[e];
+        if (r.lam) {
+            const double l = static_cast<const double *>(r.lam)[b];
+            x.x *= l;
+            x.y *= l;
+        }
+        return make_float2((float)x.x, (float)x.y);
+    } else {
+        float2 x = static_cast<const float2 *>(r.src)[e];
+        if (r.lam) {
+            const float l = static_cast<const float *>(r.lam)[b];
+            x.x *= l;
+            x.y *= l;
+        }
+        return x;
     }
 }
 
-__global__ void expand_bf16_kernel(const __nv_bfloat16 *__restrict__ compact, int planes, int chi_l, int d,
-                                   int chi_r, int Cs, int ncols, int K_pad, __nv_bfloat16 *__restrict__ B_hi,
-                                   __nv_bfloat16 *__restrict__ B_lo) {
-    const int64_t total = (int64_t)ncols * K_pad;
-    const int64_t plane = (int64_t)chi_l * d * chi_r * 2;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i / K_pad);
-        const int kappa = (int)(i - (int64_t)c * K_pad);
-        const StackedPos q = stacked_pos(c, kappa, chi_l, d, chi_r, Cs);
-        __nv_bfloat16 hi = __float2bfloat16_rn(0.f), lo = hi;
-        if (!q.zero) {
-            const int64_t e = 2 * q.cidx + (q.re_part ? 0 : 1);
-            // 16-bit values moved as bits (BF16 or FP16 planes); negation flips the sign bit of either format
-            hi = compact[e];
-            if (q.sign < 0.f) hi = __ushort_as_bfloat16((unsigned short)(__bfloat16_as_ushort(hi) ^ 0x8000u));
+// 2^floor(log2(32768 / amax)) (1 for an all-zero tensor)
+__device__ __forceinline__ float f16_site_scale(float amax) {
+    if (!(amax > 0.f)) return 1.f;
+    if (isinf(amax)) return 0.f;
+    int e;
+    const float m = frexpf(amax, &e);  // amax = m 2^e, m in [0.5, 1)
+    return ldexpf(1.f, 15 - (m == 0.5f ? e - 1 : e));
+}
+
+template <int kSource, bool kVec>
+__global__ void __launch_bounds__(256) repack16_kernel(const Repack16 r) {
+    __shared__ __align__(16) uint16_t sm[4][kRepackB][kRepackLd];  // Re hi, Im hi, Re lo, Im lo
+    const int b0 = blockIdx.x * kRepackB, a0 = blockIdx.y * kRepackA, s = blockIdx.z, tid = threadIdx.x;
+    const int planes = r.lo ? 2 : 1;
+    const float scale = r.amax ? f16_site_scale(*r.amax) : 1.f;
+    const int64_t n = (int64_t)r.chi_l * r.d * r.chi_r;
+    for (int i = tid; i < kRepackA * kRepackB; i += 256) {
+        const int a = i / kRepackB, b = i % kRepackB;
+        if (a0 + a >= r.chi_l || b0 + b >= r.chi_r) continue;
+        const int64_t e = ((int64_t)(a0 + a) * r.d + s) * r.chi_r + b0 + b;
+        if constexpr (kSource == kFrom16) {
+            const ushort2 *c = static_cast<const ushort2 *>(r.src);
+            const ushort2 hi = c[e];
+            sm[0][b][a] = hi.x;
+            sm[1][b][a] = hi.y;
             if (planes > 1) {
-                lo = compact[plane + e];
-                if (q.sign < 0.f) lo = __ushort_as_bfloat16((unsigned short)(__bfloat16_as_ushort(lo) ^ 0x8000u));
+                const ushort2 lo = c[n + e];
+                sm[2][b][a] = lo.x;
+                sm[3][b][a] = lo.y;
+            }
+        } else {
+            const float2 v = repack_value<kSource>(r, e, b0 + b);
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
+                const float x = (part ? v.y : v.x) * scale;  // exact: a power of two
+                if (r.f16) {
+                    const __half hi = __float2half_rn(x);
+                    sm[part][b][a] = __half_as_ushort(hi);
+                    if (planes > 1) sm[2 + part][b][a] = __half_as_ushort(__float2half_rn(x - __half2float(hi)));
+                } else {
+                    __nv_bfloat16 hi, lo;
+                    split_bf16(x, hi, lo);
+                    sm[part][b][a] = __bfloat16_as_ushort(hi);
+                    if (planes > 1) sm[2 + part][b][a] = __bfloat16_as_ushort(lo);
+                }
             }
         }
-        B_hi[i] = hi;
-        if (B_lo) B_lo[i] = lo;
+    }
+    __syncthreads();
+    // column (p, b) takes [Ar ; -Ai] (p = 0) or [Ai ; Ar] (p = 1) along kappa
+    for (int q = 0; q < planes; ++q) {
+        uint16_t *out = q ? r.lo : r.hi;
+        constexpr int kRun = kVec ? kRepackA / 8 : kRepackA;  // stores per run of 64
+        for (int i = tid; i < kRepackB * 4 * kRun; i += 256) {
+            const int piece = i % kRun, half = i / kRun & 1, part = i / (2 * kRun) & 1, b = i / (4 * kRun);
+            const int a = kVec ? 8 * piece : piece;
+            if (b0 + b >= r.chi_r || a0 + a >= r.chi_l) continue;
+            const uint16_t *v = &sm[2 * q + (part == half ? 0 : 1)][b][a];
+            uint16_t *dst = out + ((int64_t)s * r.Cs + part * r.chi_r + b0 + b) * r.K_pad + half * r.chi_l + a0 + a;
+            const bool negative = part == 0 && half == 1;
+            if constexpr (kVec) {
+                uint4 x = *reinterpret_cast<const uint4 *>(v);
+                const uint32_t flip = negative ? 0x80008000u : 0u;
+                *reinterpret_cast<uint4 *>(dst) = make_uint4(x.x ^ flip, x.y ^ flip, x.z ^ flip, x.w ^ flip);
+            } else {
+                *dst = (uint16_t)(*v ^ (negative ? 0x8000u : 0u));
+            }
+        }
+        // padding: the end of these columns' rows, and the outcome block's columns past 2 chi_r
+        if (a0 + kRepackA >= r.chi_l) {
+            const int pad = r.K_pad - 2 * r.chi_l;
+            for (int i = tid; i < pad * 2 * kRepackB; i += 256) {
+                const int k = i % pad, part = i / pad & 1, b = i / (2 * pad);
+                if (b0 + b < r.chi_r)
+                    out[((int64_t)s * r.Cs + part * r.chi_r + b0 + b) * r.K_pad + 2 * r.chi_l + k] = 0;
+            }
+        }
+        if (b0 + kRepackB >= r.chi_r) {
+            // 128 kappa entries per a-tile cover K_pad = roundup(2 chi_l, 64)
+            const int k0 = 2 * a0, pieces = min(2 * kRepackA, r.K_pad - k0) / 8;
+            for (int i = tid; i < (r.Cs - 2 * r.chi_r) * pieces; i += 256)
+                *reinterpret_cast<uint4 *>(out + ((int64_t)s * r.Cs + 2 * r.chi_r + i / pieces) * r.K_pad + k0 +
+                                           8 * (i % pieces)) = make_uint4(0u, 0u, 0u, 0u);
+        }
     }
 }
 
@@ -135,33 +220,32 @@ __global__ void repack_e4m3_kernel(const void *__restrict__ src, int is_f64, int
     }
 }
 
-__global__ void repack_f16_kernel(const void *__restrict__ src, int is_f64, int chi_l, int d, int chi_r, int Cs,
-                                  int ncols, int K_pad, float scale, uint16_t *__restrict__ B16,
-                                  uint16_t *__restrict__ B16_lo) {
-    const int64_t total = (int64_t)ncols * K_pad;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i / K_pad);
-        const int kappa = (int)(i - (int64_t)c * K_pad);
-        const StackedPos q = stacked_pos(c, kappa, chi_l, d, chi_r, Cs);
-        float x = 0.f;
-        if (!q.zero) x = q.sign * load_part(src, is_f64, q.cidx, q.re_part ? 0 : 1);
-        const float xs = x * scale;  // exact: a power-of-two scale
-        const __half hi = __float2half_rn(xs);
-        B16[i] = __half_as_ushort(hi);
-        if (B16_lo) B16_lo[i] = __half_as_ushort(__float2half_rn(xs - __half2float(hi)));  // the residual is exact
-    }
-}
-
-// max over |Re|, |Im| (as float) of n complex entries; non-negative floats order like their bit patterns
-__global__ void absmax_kernel(const void *__restrict__ src, int is_f64, int64_t n2, float *out) {
+// max over |Re|, |Im| (as float) of n2 / 2 complex entries, column b scaled by lam[b] (nullable); non-negative
+// floats order like their bit patterns.  One atomic per block: one per warp kept the address busy for 28 us.
+__global__ void __launch_bounds__(256) absmax_kernel(const void *__restrict__ src, int is_f64, int64_t n2, int chi_r,
+                                                     const void *__restrict__ lam, float *out) {
+    __shared__ float part[8];
     float m = 0.f;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n2; i += (int64_t)gridDim.x * blockDim.x) {
-        const float x = is_f64 ? (float)static_cast<const double *>(src)[i] : static_cast<const float *>(src)[i];
+        float x;
+        if (is_f64) {
+            double v = static_cast<const double *>(src)[i];
+            if (lam) v *= static_cast<const double *>(lam)[(i >> 1) % chi_r];
+            x = (float)v;
+        } else {
+            x = static_cast<const float *>(src)[i];
+            if (lam) x *= static_cast<const float *>(lam)[(i >> 1) % chi_r];
+        }
         m = fmaxf(m, fabsf(x));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned int *>(out), __float_as_uint(m));
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) m = fmaxf(m, part[w]);
+        atomicMax(reinterpret_cast<unsigned int *>(out), __float_as_uint(m));
+    }
 }
 
 static int grid_for(int64_t total, int block) {
@@ -171,18 +255,27 @@ static int grid_for(int64_t total, int block) {
     return (int)g;
 }
 
-void launch_repack_bf16(const void *src, int is_f64, const SiteLayout &L, __nv_bfloat16 *B_hi, __nv_bfloat16 *B_lo,
-                        cudaStream_t st) {
-    const int64_t total = (int64_t)L.ncols * L.K_pad;
-    repack_bf16_kernel<<<grid_for(total, 256), 256, 0, st>>>(src, is_f64, L.chi_l, L.d, L.chi_r, L.Cs, L.ncols,
-                                                              L.K_pad, B_hi, B_lo);
+template <int kSource>
+static void launch_repack16(const void *src, const void *lam, const float *amax, int f16, const SiteLayout &L, uint16_t *hi,
+                            uint16_t *lo, cudaStream_t st) {
+    const Repack16 r{src, lam, amax, L.chi_l, L.d, L.chi_r, L.Cs, L.K_pad, f16, hi, lo};
+    const dim3 grid((unsigned)((L.chi_r + kRepackB - 1) / kRepackB), (unsigned)((L.chi_l + kRepackA - 1) / kRepackA),
+                    (unsigned)L.d);
+    if (L.chi_l % 8 == 0) repack16_kernel<kSource, true><<<grid, 256, 0, st>>>(r);
+    else repack16_kernel<kSource, false><<<grid, 256, 0, st>>>(r);
 }
 
-void launch_expand_bf16(const __nv_bfloat16 *compact, int planes, const SiteLayout &L, __nv_bfloat16 *B_hi,
+void launch_repack_bf16(const void *src, int is_f64, const void *lam, const SiteLayout &L, __nv_bfloat16 *B_hi,
                         __nv_bfloat16 *B_lo, cudaStream_t st) {
-    const int64_t total = (int64_t)L.ncols * L.K_pad;
-    expand_bf16_kernel<<<grid_for(total, 256), 256, 0, st>>>(compact, planes, L.chi_l, L.d, L.chi_r, L.Cs, L.ncols,
-                                                              L.K_pad, B_hi, B_lo);
+    uint16_t *hi = reinterpret_cast<uint16_t *>(B_hi), *lo = reinterpret_cast<uint16_t *>(B_lo);
+    if (is_f64) launch_repack16<kFromDouble>(src, lam, nullptr, 0, L, hi, lo, st);
+    else launch_repack16<kFromFloat>(src, lam, nullptr, 0, L, hi, lo, st);
+}
+
+void launch_expand_bf16(const __nv_bfloat16 *compact, const SiteLayout &L, __nv_bfloat16 *B_hi, __nv_bfloat16 *B_lo,
+                        cudaStream_t st) {
+    launch_repack16<kFrom16>(compact, nullptr, nullptr, 0, L, reinterpret_cast<uint16_t *>(B_hi),
+                             reinterpret_cast<uint16_t *>(B_lo), st);
 }
 
 void launch_repack_e4m3(const void *src, int is_f64, const SiteLayout &L, float scale, uint8_t *B8,
@@ -192,16 +285,18 @@ void launch_repack_e4m3(const void *src, int is_f64, const SiteLayout &L, float 
                                                               L.K_pad, scale, B8);
 }
 
-void launch_repack_f16(const void *src, int is_f64, const SiteLayout &L, float scale, uint16_t *B16,
-                       uint16_t *B16_lo, cudaStream_t st) {
-    const int64_t total = (int64_t)L.ncols * L.K_pad;
-    repack_f16_kernel<<<grid_for(total, 256), 256, 0, st>>>(src, is_f64, L.chi_l, L.d, L.chi_r, L.Cs, L.ncols,
-                                                             L.K_pad, scale, B16, B16_lo);
+void launch_repack_f16(const void *src, int is_f64, const void *lam, const float *amax, const SiteLayout &L,
+                       uint16_t *B16, uint16_t *B16_lo, cudaStream_t st) {
+    if (is_f64) launch_repack16<kFromDouble>(src, lam, amax, 1, L, B16, B16_lo, st);
+    else launch_repack16<kFromFloat>(src, lam, amax, 1, L, B16, B16_lo, st);
 }
 
-void launch_absmax(const void *src, int is_f64, int64_t n_complex, float *out_dev, cudaStream_t st) {
+void launch_absmax(const void *src, int is_f64, int64_t n_complex, int chi_r, const void *lam, float *out_dev,
+                   cudaStream_t st) {
     cudaMemsetAsync(out_dev, 0, sizeof(float), st);
-    absmax_kernel<<<grid_for(2 * n_complex, 256), 256, 0, st>>>(src, is_f64, 2 * n_complex, out_dev);
+    const int64_t blocks = (2 * n_complex + 255) / 256;
+    absmax_kernel<<<(unsigned)std::min<int64_t>(blocks, 152 * 8), 256, 0, st>>>(src, is_f64, 2 * n_complex, chi_r, lam,
+                                                                             out_dev);
 }
 
 void launch_repack_f32(const void *src, int is_f64, const SiteLayout &L, float *Bt, cudaStream_t st) {

@@ -23,24 +23,27 @@ struct SiteLayout {
     int bk = 64;       // operand elements per k-block: one 128-byte swizzle row (64 BF16 or 128 FP8)
 };
 
-// ---- repack of a complex site tensor (device staging copy) -----------------
-// src: interleaved complex [chi_l][d][chi_r], float (is_f64 = 0) or double.
-// Tensor-core operand: B[c][kappa] (K-major, ld = K_pad), BF16 hi (and lo).
-void launch_repack_bf16(const void *src, int is_f64, const SiteLayout &L, __nv_bfloat16 *B_hi,
+// ---- repack of a complex site tensor ---------------------------------------
+// src: interleaved complex [chi_l][d][chi_r], float (is_f64 = 0) or double; lam (nullable, device): column b is
+// scaled by lam[b], in the input's type, first.
+// Tensor-core operand: B[c][kappa] (K-major, ld = K_pad), BF16 hi (and lo), padding zeroed.
+void launch_repack_bf16(const void *src, int is_f64, const void *lam, const SiteLayout &L, __nv_bfloat16 *B_hi,
                         __nv_bfloat16 *B_lo, cudaStream_t st);
-// Same from a compact BF16 complex copy [chi_l][d][chi_r] of (re, im) pairs
-// (planes = 1: hi only; planes = 2: hi block followed by lo block).
-void launch_expand_bf16(const __nv_bfloat16 *compact, int planes, const SiteLayout &L, __nv_bfloat16 *B_hi,
-                        __nv_bfloat16 *B_lo, cudaStream_t st);
+// Same from a compact 16-bit complex copy [chi_l][d][chi_r] of (re, im) pairs (BF16 or FP16 bits; with B_lo:
+// the hi block followed by the lo block).
+void launch_expand_bf16(const __nv_bfloat16 *compact, const SiteLayout &L, __nv_bfloat16 *B_hi, __nv_bfloat16 *B_lo,
+                        cudaStream_t st);
 // FP8 E4M3 operand B[c][kappa] (K-major, ld = K_pad bytes) of value * scale (scale a power of two).
 void launch_repack_e4m3(const void *src, int is_f64, const SiteLayout &L, float scale, uint8_t *B8,
                         cudaStream_t st);
-// Largest |Re| or |Im| of an interleaved complex tensor (as float), into *out_dev (zeroed first).
-void launch_absmax(const void *src, int is_f64, int64_t n_complex, float *out_dev, cudaStream_t st);
-// FP16 operand B[c][kappa] (K-major, ld = K_pad) of value * scale (scale a power of two), binary16 bits;
+// Largest |Re| or |Im| of an interleaved complex tensor (as float, after the scaling by lam), into *out_dev
+// (zeroed first).
+void launch_absmax(const void *src, int is_f64, int64_t n_complex, int chi_r, const void *lam, float *out_dev,
+                   cudaStream_t st);
+// FP16 operand B[c][kappa] (K-major, ld = K_pad) of value * 2^floor(log2(32768 / *amax)), binary16 bits;
 // B16_lo (optional) receives the rounding residual fp16(value * scale - B16).
-void launch_repack_f16(const void *src, int is_f64, const SiteLayout &L, float scale, uint16_t *B16,
-                       uint16_t *B16_lo, cudaStream_t st);
+void launch_repack_f16(const void *src, int is_f64, const void *lam, const float *amax, const SiteLayout &L,
+                       uint16_t *B16, uint16_t *B16_lo, cudaStream_t st);
 // FP32 SIMT operand: Bt[kappa][c] (N-major, ld = ncols), float.
 void launch_repack_f32(const void *src, int is_f64, const SiteLayout &L, float *Bt, cudaStream_t st);
 

@@ -68,8 +68,8 @@ void tune_cache_store() {
     fclose(f);
 }
 
-// Times the candidates on the staged tensor; returns bn + 10000 * mode of the fastest.
-int autotune_bn(fastmps_handle h, int chi_l, int d, int chi_r, int is_f64) {
+// Times the candidates on the tensor at src (device); returns bn + 10000 * mode of the fastest.
+int autotune_bn(fastmps_handle h, const void *src, int chi_l, int d, int chi_r, int is_f64) {
     const PrecisionPlan plan = plan_of(h->opt.precision);
     const int widest = (int)std::min<int64_t>(256, roundup(2 * (int64_t)chi_r, 32));
     const int64_t rows = 8192;
@@ -94,7 +94,7 @@ int autotune_bn(fastmps_handle h, int chi_l, int d, int chi_r, int is_f64) {
         if (!cluster)
             ok = ok && Y.ensure((size_t)rows * L.ncols * 4) && P.ensure((size_t)rows * (L.ncols / L.bn) * 4);
         if (!ok) break;
-        launch_repack_bf16(h->staging.p, is_f64, L, B[0].as<__nv_bfloat16>(),
+        launch_repack_bf16(src, is_f64, nullptr, L, B[0].as<__nv_bfloat16>(),
                            plan.b_planes > 1 ? B[1].as<__nv_bfloat16>() : nullptr, h->stream);
         __nv_bfloat16 *Vp[3] = {nullptr, nullptr, nullptr};
         for (int p = 0; p < plan.a_planes; ++p) Vp[p] = V[p].as<__nv_bfloat16>();
@@ -169,15 +169,43 @@ int autotune_bn(fastmps_handle h, int chi_l, int d, int chi_r, int is_f64) {
 
 }  // namespace
 
+// Memory of the handle's own device, at this alignment.
+static bool readable_in_place(fastmps_handle h, const void *p, size_t align) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == h->device && reinterpret_cast<uintptr_t>(p) % align == 0;
+}
+
+// Exchanges the device operands of t and `replaced`.
+static void swap_operands(Tensor &t, Tensor &replaced) {
+    using Buf = DevBuf Tensor::*;
+    for (Buf b : {&Tensor::B_hi, &Tensor::B_lo, &Tensor::Bt}) {
+        std::swap((t.*b).p, (replaced.*b).p);
+        std::swap((t.*b).bytes, (replaced.*b).bytes);
+    }
+}
+
+// Whether the operands of `from` fit layout L and are at most twice as large.
+static bool operands_fit(const Tensor &from, int precision, const SiteLayout &L) {
+    const size_t want = (size_t)L.ncols * L.K_pad * (precision == FASTMPS_FP32 ? 4 : 2);
+    auto fits = [&](const DevBuf &b) { return b.bytes >= want && b.bytes / 2 <= want; };
+    if (precision == FASTMPS_FP32) return fits(from.Bt);
+    return fits(from.B_hi) && (plan_of(precision).b_planes < 2 || fits(from.B_lo));
+}
+
+static int load_resident(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const void *src, int dtype,
+                         const void *lam_dev);
+
 int load_tensor(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const void *A, int dtype,
-                const void *lam) {
+                const void *lam, Tensor *replaced) {
     int rc = check_shape_args(h, chi_l, d, chi_r, A, dtype);
     if (rc) return rc;
     const size_t lam_bytes = (size_t)chi_r * (dtype == FASTMPS_C128 ? 8 : 4);
     t.L = make_layout(h->opt.precision, chi_l, d, chi_r);
     const int64_t nelem = (int64_t)chi_l * d * chi_r;
-    const bool tune = h->opt.autotune && is_bf16(h) && !is_fp8(h) && !is_f16(h) && h->opt.accum_chunk == 0 &&
-                      h->opt.residency == FASTMPS_RESIDENT_HBM;
     const size_t src_bytes = (size_t)nelem * (dtype == FASTMPS_C128 ? 16 : 8);
     cudaError_t e;
     const bool a_on_device = is_device_ptr(A);
@@ -234,23 +262,48 @@ int load_tensor(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const 
         }
         return FASTMPS_OK;
     }
-    if (!h->staging.ensure(src_bytes)) return fail(h, FASTMPS_ERR_OOM, "staging allocation failed");
-    e = cudaMemcpyAsync(h->staging.p, A, src_bytes, a_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                        h->stream);
-    if (e != cudaSuccess) return cuda_fail(h, e, "copy of site tensor");
+    // A tensor in this device's own memory is read in place by the 16-bit repack (which applies Lambda itself);
+    // any other is copied to the staging buffer first.
+    const bool is_f64 = dtype == FASTMPS_C128;
+    const bool repack16 = is_bf16(h) && !is_fp8(h);
+    const void *src = A;
+    if (!repack16 || !readable_in_place(h, A, is_f64 ? 16 : 8)) {
+        if (!h->staging.ensure(src_bytes)) return fail(h, FASTMPS_ERR_OOM, "staging allocation failed");
+        e = cudaMemcpyAsync(h->staging.p, A, src_bytes, a_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                            h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "copy of site tensor");
+        src = h->staging.p;
+    }
+    const void *lam_dev = nullptr;
     if (lam) {
         if (!h->lam.ensure(lam_bytes)) return fail(h, FASTMPS_ERR_OOM, "allocation failed");
         e = cudaMemcpyAsync(h->lam.p, lam, lam_bytes, is_device_ptr(lam) ? cudaMemcpyDeviceToDevice
                                                                           : cudaMemcpyHostToDevice, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "copy of Schmidt coefficients");
-        launch_scale_columns(h->staging.p, dtype == FASTMPS_C128, nelem, chi_r, h->lam.p, h->stream);
+        if (repack16) lam_dev = h->lam.p;
+        else launch_scale_columns(h->staging.p, is_f64, nelem, chi_r, h->lam.p, h->stream);
     }
+    if (!h->err.ensure(256)) return fail(h, FASTMPS_ERR_OOM, "allocation failed");
+    const bool reuse = replaced && !is_fp8(h) && !h->opt.autotune && operands_fit(*replaced, h->opt.precision, t.L);
+    if (reuse) swap_operands(t, *replaced);
+    rc = load_resident(h, t, chi_l, d, chi_r, src, dtype, lam_dev);
+    if (rc && reuse) swap_operands(t, *replaced);
+    return rc;
+}
+
+// Repack of the tensor at src (device) into t's operands.
+static int load_resident(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const void *src, int dtype,
+                         const void *lam_dev) {
+    const bool is_f64 = dtype == FASTMPS_C128;
+    const int64_t nelem = (int64_t)chi_l * d * chi_r;
+    const bool tune = h->opt.autotune && is_bf16(h) && !is_fp8(h) && !is_f16(h) && h->opt.accum_chunk == 0;
+    cudaError_t e;
     const size_t op_elems = (size_t)t.L.ncols * t.L.K_pad;
     if (is_fp8(h)) {
         // per-site power-of-two scale that puts the largest |Re|, |Im| in [224, 448]
         if (!t.B8.ensure(op_elems) || !h->err.ensure(256)) return fail(h, FASTMPS_ERR_OOM, "allocation failed");
         float amax = 0.f;
-        launch_absmax(h->staging.p, dtype == FASTMPS_C128, nelem, h->err.as<float>(), h->stream);
+        launch_absmax(h->staging.p, is_f64, nelem, chi_r, nullptr, h->err.as<float>(), h->stream);
         e = cudaMemcpyAsync(&amax, h->err.p, sizeof(float), cudaMemcpyDeviceToHost, h->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "site tensor maximum");
@@ -264,13 +317,8 @@ int load_tensor(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const 
         const bool two = plan_of(h->opt.precision).b_planes > 1;
         if (!t.B_hi.ensure(op_elems * 2) || (two && !t.B_lo.ensure(op_elems * 2)) || !h->err.ensure(256))
             return fail(h, FASTMPS_ERR_OOM, "allocation failed");
-        float amax = 0.f;
-        launch_absmax(h->staging.p, dtype == FASTMPS_C128, nelem, h->err.as<float>(), h->stream);
-        e = cudaMemcpyAsync(&amax, h->err.p, sizeof(float), cudaMemcpyDeviceToHost, h->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-        if (e != cudaSuccess) return cuda_fail(h, e, "site tensor maximum");
-        t.fp8_scale = amax > 0.f ? (float)std::exp2(std::floor(std::log2(32768.0 / (double)amax))) : 1.f;
-        launch_repack_f16(h->staging.p, dtype == FASTMPS_C128, t.L, t.fp8_scale, t.B_hi.as<uint16_t>(),
+        launch_absmax(src, is_f64, nelem, chi_r, lam_dev, h->err.as<float>(), h->stream);
+        launch_repack_f16(src, is_f64, lam_dev, h->err.as<float>(), t.L, t.B_hi.as<uint16_t>(),
                           two ? t.B_lo.as<uint16_t>() : nullptr, h->stream);
         if (!encode_2d_f16(&t.tmB[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn) ||
             (two && !encode_2d_f16(&t.tmB[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn)) ||
@@ -291,7 +339,7 @@ int load_tensor(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const 
             if (it != g_tuned.end()) {
                 code = it->second;
             } else {
-                code = autotune_bn(h, chi_l, d, chi_r, dtype == FASTMPS_C128);
+                code = autotune_bn(h, src, chi_l, d, chi_r, is_f64);
                 g_tuned[key] = code;
                 tune_cache_store();
             }
@@ -305,7 +353,7 @@ int load_tensor(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const 
             if (!t.B_lo.ensure(op_elems * 2)) return fail(h, FASTMPS_ERR_OOM, "site operand allocation failed");
             lo = t.B_lo.as<__nv_bfloat16>();
         }
-        launch_repack_bf16(h->staging.p, dtype == FASTMPS_C128, t.L, t.B_hi.as<__nv_bfloat16>(), lo, h->stream);
+        launch_repack_bf16(src, is_f64, lam_dev, t.L, t.B_hi.as<__nv_bfloat16>(), lo, h->stream);
         if (!encode_2d_bf16(&t.tmB[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn))
             return fail(h, FASTMPS_ERR_CUDA, "tensor map encoding failed");
         if (lo && !encode_2d_bf16(&t.tmB[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn))
