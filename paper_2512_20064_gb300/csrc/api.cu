@@ -106,6 +106,7 @@ int fastmps_create(fastmps_handle *out, int device, const fastmps_options *opt) 
         cudaEventCreateWithFlags(&h->contract_done[i], cudaEventDisableTiming);
         cudaEventCreateWithFlags(&h->measure_done[i], cudaEventDisableTiming);
     }
+    cudaEventCreateWithFlags(&h->prep_done, cudaEventDisableTiming);
     h->staging.host = false;
     *out = h;
     return FASTMPS_OK;
@@ -125,6 +126,7 @@ void fastmps_destroy(fastmps_handle h) {
         if (h->contract_done[i]) cudaEventDestroy(h->contract_done[i]);
         if (h->measure_done[i]) cudaEventDestroy(h->measure_done[i]);
     }
+    if (h->prep_done) cudaEventDestroy(h->prep_done);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
     if (h->measure_stream) cudaStreamDestroy(h->measure_stream);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);

@@ -375,8 +375,10 @@ extern "C" int fastmps_sample_batch(fastmps_handle runner, int count, const fast
             __nv_bfloat16 *V0[3] = {nullptr, nullptr, nullptr};
             for (int p = 0; p < a_planes; ++p) V0[p] = B.V[0][p].as<__nv_bfloat16>();
             cudaMemsetAsync(B.logp.p, 0, (size_t)P.N_pad * 8, cap);
-            launch_init_left_bf16(V0, a_planes, P.N_pad, P.ldV, cap);
-            ++launches;
+            SiteView first;
+            site_view(jobs[j].chain, 0, &first);
+            launch_init_left_bf16(V0, a_planes, P.N_pad, P.ldV, first.L.K_pad, cap);
+            launches += a_planes;
         }
         PersistentArgs g;
         g.segs = bs->segs_dev.as<PSegment>();

@@ -109,12 +109,12 @@ struct fastmps_ctx {
     fastmps::DevBuf trunc;    // device gather of the leading block of a truncated Vidal-form site
     fastmps::DevBuf disp_tab; // constants of the displacement entries for dimension disp_tab_d
     fastmps::DevBuf chain_sites;  // site table of an FP32 call that runs in one launch
-    fastmps::DevBuf disp_D, disp_u;  // per-row matrices and uniforms of one displaced micro-batch
+    fastmps::DevBuf disp_D, disp_u, disp_w;  // per-row matrices, uniforms and probability sums of one displaced micro-batch
     int disp_tab_d = 0;
     std::vector<float> disp_tab_host;
     fastmps::DevBuf slot_compact[2], slot_hi, slot_lo;  // streaming slots
     cudaEvent_t copy_done[2] = {nullptr, nullptr}, slot_free[2] = {nullptr, nullptr};
-    cudaEvent_t contract_done[2] = {nullptr, nullptr}, measure_done[2] = {nullptr, nullptr};
+    cudaEvent_t contract_done[2] = {nullptr, nullptr}, measure_done[2] = {nullptr, nullptr}, prep_done = nullptr;
     fastmps_stats stats{};
     std::vector<cudaEvent_t> ev_pool;
 };

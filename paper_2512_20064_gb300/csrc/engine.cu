@@ -203,9 +203,6 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
         // (128 rows x SMs) so that every block gets the same number of m-tiles
         const int64_t wave = (int64_t)128 * h->num_sms;
         if (bf16 && h->opt.fused_measure && !mu_dev && N2 >= wave && N_pad > N2) N2 = N2 / wave * wave;
-        // the displaced measurement reads whole scratch rows and takes a large share of a site: with at
-        // least two micro-batches it overlaps the next micro-batch's contraction on the second stream
-        if (mu_dev && N2 >= N_pad && N_pad >= 2 * wave) N2 = roundup((N_pad + 1) / 2, 128);
     }
     N2 = std::min(N2, N_pad);
     const int64_t J = (N + N2 - 1) / N2;  // micro-batches per site
@@ -222,6 +219,9 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
     // BF16 modes measure inside the contraction kernel (no second launch, one scratch buffer)
     const bool fused = bf16 && !fp8 && h->opt.fused_measure == 1 && !mu_dev;
     const int nybuf = (J > 1 && !fused) ? 2 : 1;
+    // One micro-batch per site: contraction and measurement follow each other, on one stream.  With several, a
+    // micro-batch's measurement runs on the second stream beside the next one's contraction.
+    const bool one_stream = nybuf == 1;
 
     if (ncols_max > 0 && !in_one_launch)
         for (int b = 0; b < nybuf; ++b)
@@ -273,7 +273,7 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
 
     const float *disp_tab = nullptr;
     if (mu_dev && (!(disp_tab = displacement_table(h, d)) || !h->disp_D.ensure((size_t)N2 * d * d * 8) ||
-                   !h->disp_u.ensure((size_t)N2 * 8)))
+                   !h->disp_u.ensure((size_t)N2 * 8) || !h->disp_w.ensure((size_t)N2 * 8)))
         return fail(h, FASTMPS_ERR_OOM, "displacement buffers allocation failed");
     int *d_err = h->err.as<int>();
     e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
@@ -316,25 +316,27 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
     __nv_bfloat16 *Vp[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
     for (int x = 0; x < 2; ++x)
         for (int p = 0; p < planes && bf16 && !fp8; ++p) Vp[x][p] = h->V[x][p].as<__nv_bfloat16>();
-    if (fp8) {
-        launch_init_left_e4m3(h->V[0][0].as<uint8_t>(), N_pad, ldV, st);
-        if (planes > 1) cudaMemsetAsync(h->V[0][1].p, 0, (size_t)N_pad * ldV, st);  // residual plane of [1]
-    } else if (is_f16(h))
-        launch_init_left_f16(h->V[0][0].as<uint16_t>(), h->V[0][1].as<uint16_t>(), N_pad, ldV, st);
+    // the columns that site 0 reads: a measurement writes all that the next site reads
+    const int K0 = ts[0]->L.K_pad;
+    if (fp8)
+        launch_init_left_e4m3(h->V[0][0].as<uint8_t>(), planes > 1 ? h->V[0][1].as<uint8_t>() : nullptr, N_pad, ldV, K0, st);
+    else if (is_f16(h))
+        launch_init_left_f16(h->V[0][0].as<uint16_t>(), h->V[0][1].as<uint16_t>(), N_pad, ldV, K0, st);
     else if (bf16)
-        launch_init_left_bf16(Vp[0], planes, N_pad, ldV, st);
+        launch_init_left_bf16(Vp[0], planes, N_pad, ldV, K0, st);
     else
-        launch_init_left_f32(h->V[0][0].as<float>(), N_pad, ldV, st);
-    h->stats.launches += 1;
+        launch_init_left_f32(h->V[0][0].as<float>(), N_pad, ldV, K0, st);
+    h->stats.launches += planes;
 
-    cudaStream_t ms = h->measure_stream;
+    cudaStream_t ms = one_stream ? st : h->measure_stream;
+    cudaEvent_t t_last = nullptr;  // (one stream) timing event after the last measurement
     int64_t g = 0;  // micro-batch counter over the whole call
     int64_t last_measured = -1;  // micro-batch whose measurement ran last on the measurement stream
     // the measurement stream starts after everything queued so far on the compute stream
     {
         cudaEvent_t ev = timer.get();
         cudaEventRecord(ev, st);
-        cudaStreamWaitEvent(ms, ev, 0);
+        cudaStreamWaitEvent(h->measure_stream, ev, 0);
     }
 
     // streaming: prefetch site 0
@@ -423,7 +425,8 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
             const int yb = (int)(g % nybuf);
             if (on_cluster[k]) {
                 // the rows come from the last measurement issued on the measurement stream, if any
-                if (last_measured >= 0) cudaStreamWaitEvent(st, h->measure_done[last_measured % nybuf], 0);
+                if (last_measured >= 0 && !one_stream)
+                    cudaStreamWaitEvent(st, h->measure_done[last_measured % nybuf], 0);
                 MeasureArgs ma{};
                 ma.d = d;
                 ma.chi_r = L.chi_r;
@@ -455,15 +458,14 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
                 if (e != cudaSuccess) return cuda_fail(h, e, "cluster contraction launch");
                 cudaEventRecord(c1, st);
                 timer.contract.push_back({c0, c1});
+                t_last = nullptr;
                 h->stats.launches += 1;
                 h->stats.contract_launches += 1;
                 last_measured = -1;
                 continue;
             }
-            // the scratch buffer is free once the measurement two micro-batches back is done; with one
-            // micro-batch per site the left rows of this contraction come from the previous measurement
-            if (!fused && g >= nybuf) cudaStreamWaitEvent(st, h->measure_done[yb], 0);
-            if (!fused && nybuf == 1 && g >= 1) cudaStreamWaitEvent(st, h->measure_done[0], 0);
+            // the scratch buffer is free once the measurement two micro-batches back is done
+            if (!one_stream && g >= nybuf) cudaStreamWaitEvent(st, h->measure_done[yb], 0);
             ContractOut co;
             co.Y = h->Y[yb].as<float>();
             co.ldY = L.ncols;
@@ -503,8 +505,18 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
             ma.disp_tab = disp_tab;
             ma.disp_D = mu_dev ? h->disp_D.as<float2>() : nullptr;
             ma.disp_u = mu_dev ? h->disp_u.as<double>() : nullptr;
-            cudaEvent_t c0 = timer.get(), c1 = timer.get();
-            cudaEventRecord(c0, st);
+            ma.disp_w = mu_dev ? h->disp_w.as<float2>() : nullptr;
+            if (ma.mu) {
+                // the rows' displacement matrices and uniforms depend on no outcome: they are formed on the second
+                // stream beside the contraction, after the last measurement
+                launch_displaced_prep(ma, h->measure_stream);
+                h->stats.launches += 1;
+                if (one_stream) cudaEventRecord(h->prep_done, h->measure_stream);
+            }
+            // (one stream: the event after the last measurement starts this contraction's time, unless the site's
+            // tensor is expanded in between)
+            cudaEvent_t c0 = t_last && !stream_mode ? t_last : timer.get(), c1 = timer.get();
+            if (c0 != t_last) cudaEventRecord(c0, st);
             if (bf16) {
                 ta.row0 = r0;
                 ta.rows_pad = (int)rows_pad;
@@ -524,16 +536,30 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
             cudaEventRecord(c1, st);
             timer.contract.push_back({c0, c1});
             if (!fused) {
-                cudaEvent_t m0 = timer.get(), m1 = timer.get();
-                cudaEventRecord(h->contract_done[yb], st);
-                cudaStreamWaitEvent(ms, h->contract_done[yb], 0);
-                cudaEventRecord(m0, ms);
-                if (ma.mu) launch_measure_displaced(ma, h->num_sms, ms);
+                cudaEvent_t m0 = one_stream ? c1 : timer.get(), m1 = timer.get();
+                if (one_stream) {
+                    if (ma.mu) cudaStreamWaitEvent(st, h->prep_done, 0);
+                } else {
+                    cudaEventRecord(h->contract_done[yb], st);
+                    cudaStreamWaitEvent(ms, h->contract_done[yb], 0);
+                    cudaEventRecord(m0, ms);
+                }
+                if (ma.mu) launch_measure_displaced(ma, ms);
                 else launch_measure(ma, ms);
-                h->stats.launches += ma.mu ? 2 : 1;  // the displaced measurement has a prep kernel
+                h->stats.launches += 1;
                 cudaEventRecord(m1, ms);
-                cudaEventRecord(h->measure_done[yb], ms);
+                if (ma.mu) {
+                    // the logarithms too run on the second stream, beside the next contraction
+                    if (one_stream) {
+                        cudaEventRecord(h->measure_done[0], st);
+                        cudaStreamWaitEvent(h->measure_stream, h->measure_done[0], 0);
+                    }
+                    launch_displaced_log(ma, h->measure_stream);
+                    h->stats.launches += 1;
+                }
+                if (!one_stream) cudaEventRecord(h->measure_done[yb], ms);
                 timer.measure.push_back({m0, m1});
+                t_last = one_stream ? m1 : nullptr;
                 last_measured = g;
             }
             e = cudaGetLastError();
@@ -541,7 +567,11 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
         }
     }
     // the compute stream resumes after the last measurement
-    if (last_measured >= 0) cudaStreamWaitEvent(st, h->measure_done[last_measured % nybuf], 0);
+    if (last_measured >= 0 && !one_stream) cudaStreamWaitEvent(st, h->measure_done[last_measured % nybuf], 0);
+    if (mu_dev && one_stream) {
+        cudaEventRecord(h->prep_done, h->measure_stream);
+        cudaStreamWaitEvent(st, h->prep_done, 0);
+    }
 
     // ---- outputs -------------------------------------------------------------
     if (out_samples) {

@@ -26,6 +26,11 @@ __device__ __forceinline__ f32x2 twice_f32x2(float x) {
     asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
     return d;
 }
+__device__ __forceinline__ f32x2 pack_f32x2(float x, float y) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
 __device__ __forceinline__ float2 unpack_f32x2(f32x2 v) {
     float2 r;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));

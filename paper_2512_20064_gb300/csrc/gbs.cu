@@ -34,6 +34,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "f32x2.cuh"
 #include "launch.h"
 #include "measure.cuh"
 
@@ -319,7 +320,9 @@ __device__ __forceinline__ void block_reduce_w(float (&w)[DMAX], float (*red)[DM
     }
 }
 
-// Outcome, log-probability, trace (thread 0 of the block).
+// Outcome, trace and the probability sums of the row (one thread).  The logarithm of their ratio is left to
+// displaced_log_kernel: taken here, by one lane, it cost the SM's FP64 pipe as much as 32 of them -- about a
+// thousand cycles a row, 190 us for 65536 rows, more than everything else.
 template <int DMAX>
 __device__ __forceinline__ void displaced_outputs(const MeasureArgs &a, int row, int sstar, float wsel, float Z32,
                                                   const float (&w)[DMAX]) {
@@ -327,8 +330,8 @@ __device__ __forceinline__ void displaced_outputs(const MeasureArgs &a, int row,
     const bool ok = (Z32 > 0.f) && isfinite(Z32) && (wsel > 0.f);
     const int64_t grow = a.row0 + row;
     a.outcomes[row] = (uint8_t)sstar;
-    if (ok) a.logp[grow] += log((double)wsel / (double)Z32);  // FP64 log of the FP32 sums' ratio
-    else atomicExch(a.err, (int)kDevNumeric);
+    a.disp_w[row] = ok ? make_float2(wsel, Z32) : make_float2(1.f, 1.f);
+    if (!ok) atomicExch(a.err, (int)kDevNumeric);
     const int64_t slot = a.trace ? (a.trace_slot ? (int64_t)a.trace_slot[grow] : (grow < a.trace_rows ? grow : -1))
                                  : -1;
     if (slot >= 0) {
@@ -336,6 +339,18 @@ __device__ __forceinline__ void displaced_outputs(const MeasureArgs &a, int row,
         for (int s = 0; s < DMAX; ++s)
             if (s < d) a.trace[slot * d + s] = ok ? (double)w[s] / (double)Z32 : 0.0;
     }
+}
+
+// Log-probability of each row of a measured micro-batch, one thread per row: FP64 log of the FP32 sums' ratio.
+__global__ void __launch_bounds__(128) displaced_log_kernel(const MeasureArgs a) {
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= a.rows) return;
+    const float2 w = a.disp_w[row];
+    a.logp[a.row0 + row] += log((double)w.x / (double)w.y);
+}
+
+void launch_displaced_log(const MeasureArgs &a, cudaStream_t st) {
+    if (a.rows > 0) displaced_log_kernel<<<(unsigned)((a.rows + 127) / 128), 128, 0, st>>>(a);
 }
 
 // Unstaged fallback (rows too wide for the register-resident and shared-memory variants, e.g.
@@ -443,7 +458,6 @@ __global__ void __launch_bounds__(256) measure_displaced_rows_kernel(const Measu
     block_reduce_w<DMAX>(w, red, lane, warp, T >> 5);
     float wsel, Z32;
     const int sstar = displaced_draw<DMAX>(w, d, u, wsel, Z32);
-    if (tid == 0) displaced_outputs<DMAX>(a, row, sstar, wsel, Z32, w);
     const float scale = wsel > 0.f && Z32 > 0.f && isfinite(Z32) ? rsqrtf(wsel) : 0.f;
     float2 c[DMAX];
 #pragma unroll
@@ -466,6 +480,7 @@ __global__ void __launch_bounds__(256) measure_displaced_rows_kernel(const Measu
         store_next(a, grow, chi_r + b, zi);
     }
     for (int i = 2 * chi_r + tid; i < a.K_next; i += T) store_next(a, grow, i, 0.f);
+    if (tid == 0) displaced_outputs<DMAX>(a, row, sstar, wsel, Z32, w);
 }
 
 // Vectorised variant (chi_r a multiple of 4): thread j holds the four consecutive columns
@@ -486,15 +501,24 @@ __device__ __forceinline__ void store_next4(const MeasureArgs &a, int64_t grow, 
     if (a.nplanes > 2) *reinterpret_cast<uint2 *>(a.Vp[2] + off) = *reinterpret_cast<const uint2 *>(p2);
 }
 
+// z += c y for four complex columns, two columns per packed multiply-add (each half rounded as a scalar fma):
+// zr = fma(c.x, yr, fma(-c.y, yi, zr)), zi = fma(c.x, yi, fma(c.y, yr, zi)).
 __device__ __forceinline__ void cmac4(float2 c, const float4 &yr, const float4 &yi, float4 &zr, float4 &zi) {
-    zr.x = fmaf(c.x, yr.x, fmaf(-c.y, yi.x, zr.x));
-    zr.y = fmaf(c.x, yr.y, fmaf(-c.y, yi.y, zr.y));
-    zr.z = fmaf(c.x, yr.z, fmaf(-c.y, yi.z, zr.z));
-    zr.w = fmaf(c.x, yr.w, fmaf(-c.y, yi.w, zr.w));
-    zi.x = fmaf(c.x, yi.x, fmaf(c.y, yr.x, zi.x));
-    zi.y = fmaf(c.x, yi.y, fmaf(c.y, yr.y, zi.y));
-    zi.z = fmaf(c.x, yi.z, fmaf(c.y, yr.z, zi.z));
-    zi.w = fmaf(c.x, yi.w, fmaf(c.y, yr.w, zi.w));
+    const f32x2 cx = twice_f32x2(c.x), cy = twice_f32x2(c.y), ny = twice_f32x2(-c.y);
+    const f32x2 r[2] = {pack_f32x2(yr.x, yr.y), pack_f32x2(yr.z, yr.w)};
+    const f32x2 i[2] = {pack_f32x2(yi.x, yi.y), pack_f32x2(yi.z, yi.w)};
+    f32x2 a[2] = {pack_f32x2(zr.x, zr.y), pack_f32x2(zr.z, zr.w)};
+    f32x2 b[2] = {pack_f32x2(zi.x, zi.y), pack_f32x2(zi.z, zi.w)};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        fma_f32x2(a[h], ny, i[h]);
+        fma_f32x2(a[h], cx, r[h]);
+        fma_f32x2(b[h], cy, r[h]);
+        fma_f32x2(b[h], cx, i[h]);
+    }
+    const float2 a0 = unpack_f32x2(a[0]), a1 = unpack_f32x2(a[1]), b0 = unpack_f32x2(b[0]), b1 = unpack_f32x2(b[1]);
+    zr = make_float4(a0.x, a0.y, a1.x, a1.y);
+    zi = make_float4(b0.x, b0.y, b1.x, b1.y);
 }
 
 template <int DMAX, int G>
@@ -540,7 +564,6 @@ __global__ void __launch_bounds__(256) measure_displaced_vec4_kernel(const Measu
     block_reduce_w<DMAX>(w, red, lane, warp, T >> 5);
     float wsel, Z32;
     const int sstar = displaced_draw<DMAX>(w, d, u, wsel, Z32);
-    if (tid == 0) displaced_outputs<DMAX>(a, row, sstar, wsel, Z32, w);
     const float scale = wsel > 0.f && Z32 > 0.f && isfinite(Z32) ? rsqrtf(wsel) : 0.f;
     float2 c[DMAX];
 #pragma unroll
@@ -562,46 +585,61 @@ __global__ void __launch_bounds__(256) measure_displaced_vec4_kernel(const Measu
     }
     for (int i = 2 * chi_r + 4 * tid; i < a.K_next; i += 4 * T)
         store_next4(a, grow, i, make_float4(0.f, 0.f, 0.f, 0.f));
+    if (tid == 0) displaced_outputs<DMAX>(a, row, sstar, wsel, Z32, w);
 }
 
-// Narrow rows (d * chi_r <= 2048, chi_r a multiple of 4): one warp per row, the row's d blocks
-// copied to shared memory with cp.async (16-byte chunks, all in flight at once) instead of registers,
-// so that about 28 rows per SM are in flight (shared memory bounds it, not registers).
+// Narrow rows (d * chi_r <= 2048, chi_r a multiple of 4): one warp per row, the row's d blocks and its matrix
+// copied to shared memory with cp.async (all in flight at once) instead of registers, so that about 25 rows per
+// SM are in flight (shared memory bounds it, not registers).  Bound by HBM: 65536 rows (d = 4, chi = 256, BF16
+// planes) 108 us = 6.3 TB/s, 190 us before the logarithm was left to displaced_log_kernel.  Warps that walk over
+// the rows with two buffers each, half as many, take 140-146 us.
 template <int DMAX>
 __global__ void __launch_bounds__(32) measure_displaced_smem_kernel(const MeasureArgs a) {
-    extern __shared__ __align__(16) float srow[];  // d blocks of [Re (chi_r) | Im (chi_r)]
+    extern __shared__ __align__(16) float srow[];  // d blocks of [Re (chi_r) | Im (chi_r)], then the matrix
     const int row = blockIdx.x, lane = threadIdx.x;
     const int d = a.d, chi_r = a.chi_r, nf2 = 2 * chi_r, ngroups = chi_r >> 2, dd = d * d;
     const int64_t Cs = a.Cs;
     const float *yrow = a.Y + (int64_t)row * a.ldY;
+    const float2 *D = reinterpret_cast<const float2 *>(srow + d * nf2);
     {
-        const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(srow);
+        const uint32_t sbase = smem_u32(srow);
+        const float2 *Drow = a.disp_D + (int64_t)row * dd;
+        for (int e = lane; e < dd; e += 32)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sbase + 4u * (uint32_t)(d * nf2 + 2 * e)),
+                         "l"(Drow + e)
+                         : "memory");
         for (int t = 0; t < d; ++t)
             for (int i = lane * 4; i < nf2; i += 128)
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sbase + 4u * (uint32_t)(t * nf2 + i)),
                              "l"(yrow + t * Cs + i)
                              : "memory");
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        cp_async_commit();
     }
-    const float2 *Drow = a.disp_D + (int64_t)row * dd;
     const double u = a.disp_u[row];
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    cp_async_wait<0>();
     __syncwarp();
     const float4 *s4 = reinterpret_cast<const float4 *>(srow);
     const int q = nf2 >> 2;  // float4 per block
     float w[DMAX];
 #pragma unroll
-    for (int s = 0; s < DMAX; ++s) {
-        w[s] = 0.f;
-        if (s >= d) continue;
-        float2 c[DMAX];
+    for (int s = 0; s < DMAX; ++s) w[s] = 0.f;
+    for (int g = lane; g < ngroups; g += 32) {
+        // the group's d blocks stay in registers over all outcomes (read again for each, they took the larger part
+        // of the shared-memory bandwidth)
+        float4 yr[DMAX], yi[DMAX];
 #pragma unroll
-        for (int t = 0; t < DMAX; ++t) c[t] = t < d ? Drow[s * d + t] : make_float2(0.f, 0.f);
-        for (int g = lane; g < ngroups; g += 32) {
+        for (int t = 0; t < DMAX; ++t) {
+            if (t >= d) break;
+            yr[t] = s4[t * q + g];
+            yi[t] = s4[t * q + ngroups + g];
+        }
+#pragma unroll
+        for (int s = 0; s < DMAX; ++s) {
+            if (s >= d) break;
             float4 zr = make_float4(0.f, 0.f, 0.f, 0.f), zi = zr;
 #pragma unroll
             for (int t = 0; t < DMAX; ++t)
-                if (t < d) cmac4(c[t], s4[t * q + g], s4[t * q + ngroups + g], zr, zi);
+                if (t < d) cmac4(D[s * d + t], yr[t], yi[t], zr, zi);
             w[s] += zr.x * zr.x + zr.y * zr.y + zr.z * zr.z + zr.w * zr.w + zi.x * zi.x + zi.y * zi.y +
                     zi.z * zi.z + zi.w * zi.w;
         }
@@ -609,12 +647,11 @@ __global__ void __launch_bounds__(32) measure_displaced_smem_kernel(const Measur
     block_reduce_w<DMAX>(w, nullptr, lane, 0, 1);
     float wsel, Z32;
     const int sstar = displaced_draw<DMAX>(w, d, u, wsel, Z32);
-    if (lane == 0) displaced_outputs<DMAX>(a, row, sstar, wsel, Z32, w);
     const float scale = wsel > 0.f && Z32 > 0.f && isfinite(Z32) ? rsqrtf(wsel) : 0.f;
     float2 c[DMAX];
 #pragma unroll
     for (int t = 0; t < DMAX; ++t) {
-        const float2 e = t < d ? Drow[sstar * d + t] : make_float2(0.f, 0.f);
+        const float2 e = t < d ? D[sstar * d + t] : make_float2(0.f, 0.f);
         c[t] = make_float2(e.x * scale, e.y * scale);
     }
     const int64_t grow = a.row0 + row;
@@ -628,6 +665,7 @@ __global__ void __launch_bounds__(32) measure_displaced_smem_kernel(const Measur
     }
     for (int i = 2 * chi_r + 4 * lane; i < a.K_next; i += 128)
         store_next4(a, grow, i, make_float4(0.f, 0.f, 0.f, 0.f));
+    if (lane == 0) displaced_outputs<DMAX>(a, row, sstar, wsel, Z32, w);
 }
 
 template <int DMAX>
@@ -636,7 +674,7 @@ bool launch_smem_variant(const MeasureArgs &a, cudaStream_t st) {
         return false;
     } else {
         if ((a.chi_r & 3) || (a.K_next & 3) || (a.ld_next & 3) || a.d * a.chi_r > 2048) return false;
-        const size_t smem = (size_t)a.d * 2 * a.chi_r * sizeof(float);
+        const size_t smem = ((size_t)a.d * 2 * a.chi_r + 2 * (size_t)a.d * a.d) * sizeof(float);
         measure_displaced_smem_kernel<DMAX><<<(unsigned)a.rows, 32, smem, st>>>(a);
         return true;
     }
@@ -703,13 +741,16 @@ void launch_displaced_variant(const MeasureArgs &a, cudaStream_t st) {
     measure_displaced_kernel<DMAX><<<grid, DISP_WARPS * 32, 0, st>>>(a);
 }
 
-void launch_measure_displaced(const MeasureArgs &a, int num_sms, cudaStream_t st) {
-    (void)num_sms;
+void launch_displaced_prep(const MeasureArgs &a, cudaStream_t st) {
     if (a.rows <= 0) return;
     const unsigned pg = (unsigned)((a.rows + 255) / 256);
     if (a.d <= 4) displaced_prep_kernel<4><<<pg, 256, 0, st>>>(a);
     else if (a.d <= 8) displaced_prep_kernel<8><<<pg, 256, 0, st>>>(a);
     else displaced_prep_kernel<kMaxDisplacedD><<<pg, 256, 0, st>>>(a);
+}
+
+void launch_measure_displaced(const MeasureArgs &a, cudaStream_t st) {
+    if (a.rows <= 0) return;
     if (a.d <= 4) launch_displaced_variant<4>(a, st);
     else if (a.d <= 8) launch_displaced_variant<8>(a, st);
     else launch_displaced_variant<kMaxDisplacedD>(a, st);

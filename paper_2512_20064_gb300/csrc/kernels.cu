@@ -73,7 +73,7 @@ __device__ __forceinline__ StackedPos stacked_pos(int c, int kappa, int chi_l, i
 // The operand is the transpose of the tensor's rows: a block reads 64 x 32 entries (a, b) of one outcome along b,
 // keeps them as 16-bit values in shared memory, and writes the four runs of 64 entries along kappa that they make
 // (16-byte stores where chi_l is a multiple of 8).  Reading one entry per stored value along kappa instead, a
-// chi_r-strided gather, took 185 us for chi = 2000, d = 3.
+// chi_r-strided gather, took 185 us for chi = 2000, d = 3; this takes 44 (144 MB).
 struct Repack16 {
     const void *src;       // [chi_l][d][chi_r] complex
     const void *lam;       // [chi_r] real, or null
@@ -308,53 +308,38 @@ void launch_repack_f32(const void *src, int is_f64, const SiteLayout &L, float *
 // ---------------------------------------------------------------------------
 // Left boundary v_0 = [1]: row = [1, 0, ..., 0] (real part 1, imaginary 0).
 // ---------------------------------------------------------------------------
-__global__ void init_left_bf16_kernel(__nv_bfloat16 *V0, __nv_bfloat16 *V1, __nv_bfloat16 *V2, int64_t rows,
-                                      int ld) {
-    const int64_t total = rows * ld;
+// One 16-byte piece per thread; `one` is the bit pattern of 1 in column 0 (little-endian, in the first bytes).
+__global__ void init_left_kernel(uint4 *__restrict__ V, int64_t rows, int ld, int cols, uint32_t one) {
+    const int64_t total = rows * cols;  // ld, cols: in pieces
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const bool one = (i % ld) == 0;
-        V0[i] = __float2bfloat16_rn(one ? 1.f : 0.f);
-        V1[i] = __float2bfloat16_rn(0.f);
-        if (V2) V2[i] = __float2bfloat16_rn(0.f);
+        const int64_t r = i / cols;
+        const int c = (int)(i - r * cols);
+        V[r * ld + c] = make_uint4(c == 0 ? one : 0u, 0u, 0u, 0u);
     }
 }
 
-__global__ void init_left_f32_kernel(float *V, int64_t rows, int ld) {
-    const int64_t total = rows * ld;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-        V[i] = (i % ld) == 0 ? 1.f : 0.f;
+static void init_left_plane(void *V, int64_t rows, int ld, int cols, int elem_bytes, uint32_t one, cudaStream_t st) {
+    const int per = 16 / elem_bytes;  // ld and cols are multiples of 64
+    init_left_kernel<<<grid_for(rows * (cols / per), 256), 256, 0, st>>>(static_cast<uint4 *>(V), rows, ld / per,
+                                                                          cols / per, one);
 }
 
-__global__ void init_left_e4m3_kernel(uint8_t *V8, int64_t rows, int ld) {
-    const int64_t total = rows * ld;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-        V8[i] = (uint8_t)__nv_cvt_float_to_fp8((i % ld) == 0 ? 1.f : 0.f, __NV_SATFINITE, __NV_E4M3);
+void launch_init_left_f16(uint16_t *V0, uint16_t *V1, int64_t rows, int ld, int cols, cudaStream_t st) {
+    init_left_plane(V0, rows, ld, cols, 2, 0x3C00u, st);
+    init_left_plane(V1, rows, ld, cols, 2, 0u, st);
 }
 
-__global__ void init_left_f16_kernel(uint16_t *V0, uint16_t *V1, int64_t rows, int ld) {
-    const int64_t total = rows * ld;
-    const uint16_t one = __half_as_ushort(__float2half_rn(1.f)), zero = __half_as_ushort(__float2half_rn(0.f));
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        V0[i] = (i % ld) == 0 ? one : zero;
-        V1[i] = zero;
-    }
+void launch_init_left_e4m3(uint8_t *V8, uint8_t *V8lo, int64_t rows, int ld, int cols, cudaStream_t st) {
+    init_left_plane(V8, rows, ld, cols, 1, 0x38u, st);
+    if (V8lo) init_left_plane(V8lo, rows, ld, cols, 1, 0u, st);
 }
 
-void launch_init_left_f16(uint16_t *V0, uint16_t *V1, int64_t rows, int ld, cudaStream_t st) {
-    init_left_f16_kernel<<<grid_for(rows * ld, 256), 256, 0, st>>>(V0, V1, rows, ld);
+void launch_init_left_bf16(__nv_bfloat16 *const *Vp, int nplanes, int64_t rows, int ld, int cols, cudaStream_t st) {
+    for (int p = 0; p < nplanes; ++p) init_left_plane(Vp[p], rows, ld, cols, 2, p ? 0u : 0x3F80u, st);
 }
 
-void launch_init_left_e4m3(uint8_t *V8, int64_t rows, int ld, cudaStream_t st) {
-    init_left_e4m3_kernel<<<grid_for(rows * ld, 256), 256, 0, st>>>(V8, rows, ld);
-}
-
-void launch_init_left_bf16(__nv_bfloat16 *const *Vp, int nplanes, int64_t rows, int ld, cudaStream_t st) {
-    init_left_bf16_kernel<<<grid_for(rows * ld, 256), 256, 0, st>>>(Vp[0], Vp[1], nplanes > 2 ? Vp[2] : nullptr,
-                                                                      rows, ld);
-}
-
-void launch_init_left_f32(float *V, int64_t rows, int ld, cudaStream_t st) {
-    init_left_f32_kernel<<<grid_for(rows * ld, 256), 256, 0, st>>>(V, rows, ld);
+void launch_init_left_f32(float *V, int64_t rows, int ld, int cols, cudaStream_t st) {
+    init_left_plane(V, rows, ld, cols, 4, 0x3F800000u, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -48,12 +48,12 @@ void launch_repack_f16(const void *src, int is_f64, const void *lam, const float
 void launch_repack_f32(const void *src, int is_f64, const SiteLayout &L, float *Bt, cudaStream_t st);
 
 // ---- left operand ----------------------------------------------------------
-// Set rows [0, rows) of V to the boundary vector v_0 = [1] (row = [1, 0, ... 0], ld elements).
-void launch_init_left_bf16(__nv_bfloat16 *const *Vp, int nplanes, int64_t rows, int ld, cudaStream_t st);
-void launch_init_left_f32(float *V, int64_t rows, int ld, cudaStream_t st);
-void launch_init_left_e4m3(uint8_t *V8, int64_t rows, int ld, cudaStream_t st);
-// FP16 planes of v_0 = [1]: plane 0 holds 1.0 in column 0, plane 1 zeros.
-void launch_init_left_f16(uint16_t *V0, uint16_t *V1, int64_t rows, int ld, cudaStream_t st);
+// Set columns [0, cols) of rows [0, rows) of V (leading dimension ld) to the boundary vector v_0 = [1]: 1 in
+// column 0 of plane 0, else 0.
+void launch_init_left_bf16(__nv_bfloat16 *const *Vp, int nplanes, int64_t rows, int ld, int cols, cudaStream_t st);
+void launch_init_left_f32(float *V, int64_t rows, int ld, int cols, cudaStream_t st);
+void launch_init_left_e4m3(uint8_t *V8, uint8_t *V8lo, int64_t rows, int ld, int cols, cudaStream_t st);
+void launch_init_left_f16(uint16_t *V0, uint16_t *V1, int64_t rows, int ld, int cols, cudaStream_t st);
 
 // ---- contraction kernels ---------------------------------------------------
 struct ContractOut {
@@ -167,6 +167,7 @@ struct MeasureArgs {
     const float *disp_tab = nullptr;   // displaced measurement: constants of the displacement entries
     float2 *disp_D = nullptr;          // displaced measurement: per-row matrices [row][d*d] (prep kernel output)
     double *disp_u = nullptr;          // displaced measurement: per-row uniforms (prep kernel output)
+    float2 *disp_w = nullptr;          // displaced measurement: per-row (w_{s*}, Z) for launch_displaced_log
     uint8_t *outcomes;        // [rows] outcome bytes of this site (site-major buffer slice)
     double *logp;             // [rows] accumulated log-probability
     double *trace;            // nullable: [trace_rows][d] normalised conditionals of this site
@@ -188,9 +189,13 @@ void build_displacement_table(int d, float *tab /* d * d * (2d + 1) */);
 void launch_displacement(const float2 *mu, int64_t N, int d, const float *tab, float2 *D, int num_sms,
                          cudaStream_t st);
 // Measurement with the physical index of each row mixed by D(a.mu[row]) first (a.mu != nullptr,
-// d <= kMaxDisplacedD, FP32 or BF16-plane next rows).  Launches a prep kernel (one thread per row:
-// the row's matrix and uniform into a.disp_D / a.disp_u) and the measurement kernel.
-void launch_measure_displaced(const MeasureArgs &a, int num_sms, cudaStream_t st);
+// d <= kMaxDisplacedD, FP32 or BF16-plane next rows), after launch_displaced_prep (one thread per row: the row's
+// matrix and uniform into a.disp_D / a.disp_u; reads a.mu only).
+void launch_displaced_prep(const MeasureArgs &a, cudaStream_t st);
+void launch_measure_displaced(const MeasureArgs &a, cudaStream_t st);
+// Adds log(w_{s*} / Z) of the measured rows to their log-probabilities (after launch_measure_displaced, before the
+// next one of the same scratch).
+void launch_displaced_log(const MeasureArgs &a, cudaStream_t st);
 
 // Self-test: one bounded mbarrier wait that nothing completes (status, device time waited).
 void launch_bounded_wait_selftest(uint64_t limit_ns, int *status, unsigned long long *waited_ns, cudaStream_t st);

@@ -98,7 +98,7 @@ int autotune_bn(fastmps_handle h, const void *src, int chi_l, int d, int chi_r, 
                            plan.b_planes > 1 ? B[1].as<__nv_bfloat16>() : nullptr, h->stream);
         __nv_bfloat16 *Vp[3] = {nullptr, nullptr, nullptr};
         for (int p = 0; p < plan.a_planes; ++p) Vp[p] = V[p].as<__nv_bfloat16>();
-        launch_init_left_bf16(Vp, plan.a_planes, rows, L.K_pad, h->stream);  // every row the vector [1, 0, ...]
+        launch_init_left_bf16(Vp, plan.a_planes, rows, L.K_pad, L.K_pad, h->stream);  // every row the vector [1, 0, ...]
         cudaMemsetAsync(err.p, 0, sizeof(int), h->stream);
         TcArgs ta;
         ta.a_planes = plan.a_planes;

@@ -171,8 +171,10 @@ extern "C" int fastmps_sample_noalloc(fastmps_handle h, int M, int d, const int 
     cudaError_t e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(logp, 0, (size_t)N_pad * 8, st);
     if (e != cudaSuccess) return set_error(h, FASTMPS_ERR_CUDA, "cudaMemsetAsync failed");
-    if (bf16) launch_init_left_bf16(Vp[0], planes, N_pad, ldV, st);
-    else launch_init_left_f32(V32[0], N_pad, ldV, st);
+    SiteView first;
+    site_view(h, 0, &first);
+    if (bf16) launch_init_left_bf16(Vp[0], planes, N_pad, ldV, first.L.K_pad, st);
+    else launch_init_left_f32(V32[0], N_pad, ldV, first.L.K_pad, st);
 
     for (int k = 0; k < M; ++k) {
         SiteView sv, sv_next;

@@ -76,3 +76,26 @@ def test_batched_measurements_at_their_edges(precision):
         a, l = s.sample(j["bonds"], j["d"], j["N"], j["seed"], n0=j["n0"], job=j["job"])
         assert np.array_equal(a, j["out_samples"]) and np.array_equal(l, j["out_logprob"])
         s.close()
+
+
+@pytest.mark.parametrize("precision,d,chi", [("bf16x2", 4, 20), ("fp32", 4, 17), ("bf16x2", 3, 700), ("fp32", 9, 12),
+                                             ("bf16x2", 8, 256), ("fp32", 16, 6)])
+def test_displaced_micro_batches_give_the_same_bits(precision, d, chi):
+    """Displaced rows in one micro-batch per site (one stream; matrices and logarithms beside the contraction) and
+    in several (two streams), for each variant of the measurement: bit for bit the same, and within tolerance of
+    the oracle."""
+    import paper_2512_20064_gb300 as F
+
+    M, N = 6, 300
+    b, ts, _ = gen.mps_tensors(M, d, chi, base_seed=15, skew=1.5, dtype=np.complex64)
+    mu = gen.gbs_amplitudes(M, N, 0.4, seed=8)
+    out = []
+    for mb in (0, 128):
+        with F.Sampler(precision=precision, max_microbatch=mb) as s:
+            s.load_chain(ts)
+            for _ in range(2):  # a second call finds the buffers of the first
+                out.append(s.sample(b, d, N, 6, mu=mu, trace_rows=N))
+    for o in out[1:]:
+        assert all(np.array_equal(x, y) for x, y in zip(out[0], o))
+    smp, lp, tr = out[0]
+    parity.check(b, _stored(ts, precision), 6, np.arange(N), smp, lp, TOL[precision], dev_trace=tr, trace_rows=N, mu=mu)
