@@ -378,7 +378,8 @@ struct F32Tile {
     static constexpr int BK = TM == 8 ? 8 : 16;    // K entries per stage
     static constexpr int AK = BK * BM / F32_THREADS;  // left entries per thread and stage, along K
     static constexpr int RG = TM == 8 ? 4 : TM;    // consecutive rows per thread; TM = 8: again 64 rows on
-    static constexpr size_t bytes = sizeof(float) * (2 * BK * (BM + F32_BN) + BM * F32_BN);
+    static constexpr int floats = 2 * BK * (BM + F32_BN) + BM * F32_BN;
+    static constexpr size_t bytes = sizeof(float) * floats + 16;  // + the tile's place, for the epilogue
 };
 
 // One (16 TM) x (64 NQ) tile.  Thread (ty, tx) holds rows 64 g + RG ty + .. and columns 64 q + 4 tx .. + 3.
@@ -386,7 +387,7 @@ template <int TM, int NQ>
 __device__ __forceinline__ void contract_f32_tile(const float *__restrict__ Ag, int64_t ldV,
                                                   const float *__restrict__ Bg, int ldB, int K,
                                                   float *__restrict__ Y, int64_t ldY, float *__restrict__ P, int ldP,
-                                                  int rows_left, float *smem) {
+                                                  int rows_valid, float *smem) {
     using T = F32Tile<TM>;
     constexpr int BM = T::BM, BK = T::BK, AK = T::AK, RG = T::RG, NP = TM / 2, NC = 4 * NQ;
     float *As = smem;                                // [2][BK][BM]
@@ -510,6 +511,11 @@ __device__ __forceinline__ void contract_f32_tile(const float *__restrict__ Ag, 
         }
     }
 
+    // (the tile's place is read back here, so that it takes no registers from the loop)
+    const int *place = reinterpret_cast<const int *>(smem + T::floats);
+    const int m0 = place[0] * BM, rows_left = rows_valid - m0;
+    Y += (int64_t)m0 * ldY + (int64_t)place[1] * F32_BN;
+    P += (int64_t)m0 * ldP + place[1];
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int r = 64 * (i / RG) + ty * RG + i % RG;
@@ -538,17 +544,32 @@ template <int TM>
 __global__ void __launch_bounds__(F32_THREADS, 2)
 contract_f32_kernel(const float *__restrict__ V, int64_t ldV, int64_t row0, const float *__restrict__ Bt, int ldB,
                     int K, float *__restrict__ Y, int64_t ldY, float *__restrict__ P, int ldP, int rows_valid,
-                    int tiles_per_s, int nreal) {
+                    int tiles_per_s, int nreal, int num_m) {
     extern __shared__ __align__(16) float f32_smem[];
     constexpr int BM = F32Tile<TM>::BM;
-    const int64_t m0 = (int64_t)blockIdx.y * BM;
-    const int n0 = blockIdx.x * F32_BN;
-    const int cols = nreal - (int)(blockIdx.x % tiles_per_s) * F32_BN;  // columns of the tile that are not padding
-    const float *Ag = V + (row0 + m0) * ldV;
-    float *Yt = Y + m0 * ldY + n0, *Pt = P + m0 * ldP + blockIdx.x;
-    const int left = rows_valid - (int)m0;
-    if (cols > 64) contract_f32_tile<TM, 2>(Ag, ldV, Bt + n0, ldB, K, Yt, ldY, Pt, ldP, left, f32_smem);
-    else contract_f32_tile<TM, 1>(Ag, ldV, Bt + n0, ldB, K, Yt, ldY, Pt, ldP, left, f32_smem);
+    // Tiles with 64 padding columns (the last of each outcome, `half` of them per row of tiles) cost half of the
+    // others and come last: an SM that has a whole tile gets a half one with it.  In the order of the columns some
+    // SMs got two whole tiles and others two half ones (d = 6, chi = 90, 3001 rows, 288 tiles: 32 sites in 1.74 ms,
+    // 1.95 in that order).
+    const int T = tiles_per_s, nx = ldB / F32_BN, half = nreal - (T - 1) * F32_BN <= 64 ? nx / T : 0;
+    const int whole = nx - half, id = blockIdx.x, first_half = whole * num_m;
+    int m, n;
+    if (id < first_half) {
+        m = id / whole;
+        const int j = id - m * whole;
+        n = half ? j / (T - 1) * T + j % (T - 1) : j;
+    } else {
+        m = (id - first_half) / half;
+        n = (id - first_half - m * half) * T + T - 1;
+    }
+    if (threadIdx.x == 0) {
+        int *place = reinterpret_cast<int *>(f32_smem + F32Tile<TM>::floats);
+        place[0] = m;
+        place[1] = n;
+    }
+    const float *Ag = V + (row0 + (int64_t)m * BM) * ldV, *Bg = Bt + (int64_t)n * F32_BN;
+    if (id < first_half) contract_f32_tile<TM, 2>(Ag, ldV, Bg, ldB, K, Y, ldY, P, ldP, rows_valid, f32_smem);
+    else contract_f32_tile<TM, 1>(Ag, ldV, Bg, ldB, K, Y, ldY, P, ldP, rows_valid, f32_smem);
 }
 
 void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, const float *Bt, const SiteLayout &L,
@@ -563,9 +584,10 @@ void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, const float 
         auto kern = contract_f32_kernel<decltype(tm)::value>;
         if (T::bytes > 48 * 1024)
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::bytes);
-        const dim3 grid((unsigned)nx, (unsigned)((o.rows_valid + T::BM - 1) / T::BM));
-        kern<<<grid, F32_THREADS, T::bytes, st>>>(V, ldV, row0, Bt, L.ncols, L.K_pad, o.Y, o.ldY, o.P, o.ldP,
-                                                  o.rows_valid, L.tiles_per_s, 2 * L.chi_r);
+        const int64_t num_m = (o.rows_valid + T::BM - 1) / T::BM;
+        kern<<<(unsigned)(nx * num_m), F32_THREADS, T::bytes, st>>>(V, ldV, row0, Bt, L.ncols, L.K_pad, o.Y, o.ldY, o.P,
+                                                                    o.ldP, o.rows_valid, L.tiles_per_s, 2 * L.chi_r,
+                                                                    (int)num_m);
     };
     if (nx * ((o.rows_valid + 31) / 32) <= 152) run(std::integral_constant<int, 2>());
     else if (nx * ((o.rows_valid + 63) / 64) <= 152) run(std::integral_constant<int, 4>());

@@ -99,3 +99,20 @@ def test_displaced_micro_batches_give_the_same_bits(precision, d, chi):
         assert all(np.array_equal(x, y) for x, y in zip(out[0], o))
     smp, lp, tr = out[0]
     parity.check(b, _stored(ts, precision), 6, np.arange(N), smp, lp, TOL[precision], dev_trace=tr, trace_rows=N, mu=mu)
+
+
+@pytest.mark.parametrize("d", [2, 4, 5, 8])
+def test_displacement_pairs_and_singles_give_the_same_bits(d):
+    """Two samples per thread (even counts, aligned arrays) against one (odd counts, 8-byte aligned arrays)."""
+    import torch
+
+    import paper_2512_20064_gb300 as F
+
+    mu = torch.from_numpy(gen.gbs_amplitudes(1, 771, 0.6, seed=3)[0]).cuda()
+    with F.Sampler() as s:
+        ref = s.displacement(mu, d)  # 771: singles
+        for n in (1, 2, 512, 770):
+            assert np.array_equal(s.displacement(mu[:n], d), ref[:, :, :n])
+            shifted = torch.empty(d * d * n + 1, dtype=torch.complex64, device="cuda")[1:]
+            F.fastmps_displacement(s.h, mu[:n], d, out=shifted)
+            assert np.array_equal(shifted.cpu().numpy().reshape(d, d, n), ref[:, :, :n])
