@@ -420,6 +420,10 @@ void precision_products(int precision, int *a_planes, int *b_planes, int *nprod,
     }
 }
 
+bool encode_scratch_map(CUtensorMap *map, const void *base, uint64_t cols, uint64_t rows, uint64_t ld_elems) {
+    return encode_2d_f32_scratch(map, base, cols, rows, ld_elems);
+}
+
 bool encode_bf16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint64_t ld_elems,
                      uint32_t box_outer) {
     return encode_2d_bf16(map, base, inner, outer, ld_elems, 64, box_outer);

@@ -302,15 +302,15 @@ extern "C" int fastmps_sample_batch(fastmps_handle runner, int count, const fast
                 S.done_base = done;
                 // fixed row strides (the job's widest site): m-tiles of consecutive steps run
                 // concurrently, so a row's scratch must not move when the site's width changes
-                S.Y = B.Y.as<float>();
-                S.ldY = P.ncols_max;
+                if (!encode_scratch_map(&S.tmY, B.Y.p, L.ncols, rows, P.ncols_max))
+                    return set_error(runner, FASTMPS_ERR_CUDA, "tensor map encoding failed");
                 S.P = B.P.as<float>();
                 S.ldP = P.ldP_max;
                 S.rows_valid = (int)rows;
                 MeasureArgs &m = hm[si];
                 m = MeasureArgs{};
-                m.Y = S.Y;
-                m.ldY = S.ldY;
+                m.Y = B.Y.as<float>();
+                m.ldY = P.ncols_max;
                 m.P = S.P;
                 m.ldP = S.ldP;
                 m.d = J.d;

@@ -408,6 +408,34 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)
         : "memory");
 }
 
+constexpr uint32_t kYWarpBytes = 4096;  // a warp's 32 x 32 FP32 chunk of the scratch
+
+// ---------------------------------------------------------------------------
+// Scratch stores.  A warp stages the 32 rows x 32 columns it read from tensor memory in a buffer of its own
+// (128-byte rows, the 128-byte swizzle that the tensor map expects) and its first lane stores them with TMA; no
+// other warp is waited for.  With one 128-row store for four warps, two barriers per 32 columns made the
+// epilogue of a 128 x 256 tile 12 thousand cycles long -- longer than its products at K = 512 (8 thousand).
+// two_buffers: the caller alternates between two buffers, so one earlier store may still be reading.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void stage_and_store(const CUtensorMap *tmY, uint8_t *buf, const uint32_t (&r)[32], int lane,
+                                                int x, int y, int rows_valid, bool two_buffers) {
+    if (lane == 0) {
+        if (two_buffers) bulk_wait_read_1();
+        else bulk_wait_read_0();
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        *reinterpret_cast<uint4 *>(buf + lane * 128 + ((j ^ (lane & 7)) * 16)) =
+            make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0 && y < rows_valid) {
+        tma_store_2d(tmY, buf, x, y);
+        bulk_commit();
+    }
+}
+
 // Shared-memory matrix descriptor for a K-major operand tile stored with the
 // 128-byte swizzle: rows of 64 BF16 (128 B), 8-row groups 1024 B apart.
 // Fields: start address >> 4 (bits 0-13), leading byte offset >> 4 (16-29,

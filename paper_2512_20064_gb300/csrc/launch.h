@@ -213,6 +213,7 @@ namespace fastmps {
 struct PSegment {  // 64-byte aligned through its CUtensorMap members
     CUtensorMap tmA[3];
     CUtensorMap tmB[2];
+    CUtensorMap tmY;     // the job's scratch, rows of this chunk: boxes of 32 columns x 32 rows
     int64_t task_begin;
     int num_m_tiles, num_n_tiles, num_k_blocks, bn;
     uint32_t idesc, tx_bytes;
@@ -220,8 +221,6 @@ struct PSegment {  // 64-byte aligned through its CUtensorMap members
     int step;            // c * M + k: steps every m-tile of this chunk has been measured for before this segment
     int64_t slot_base;   // measured[slot_base + mt]: 32-row measurements completed by m-tile slot mt of the job
     int64_t done_base;   // tiles_done[done_base + mt]: finished tiles of m-tile mt of this segment
-    float *Y;
-    int64_t ldY;
     float *P;
     int ldP;
     int rows_valid;

@@ -67,7 +67,6 @@ constexpr int kThreadsFused = 320;           // + 4 measurement warps
 constexpr int kRing = 4;                     // finished m-tiles queued for the measurement warps
 constexpr int kBarrierBytes = 2048;          // mbarriers, ring, measurement staging
 constexpr uint32_t kYStageBytes = 16384;     // one 128 x 32 FP32 chunk of the scratch tile (two buffers)
-constexpr uint32_t kYWarpBytes = 4096;       // a warp's 32 rows of it
 constexpr uint32_t kTmemCols = 512;          // 2 accumulators x 256 columns
 constexpr uint32_t kAccStride = 256;
 constexpr uint32_t kATileBytes = kBM * kBK * 2;  // 16 KB
@@ -351,32 +350,6 @@ template <bool kPair>
 __device__ __forceinline__ void release_accumulator(uint64_t *tempty) {
     if (kPair) mbar_arrive_cluster(mapa_shared(smem_u32(tempty), 0));
     else mbar_arrive(tempty);
-}
-
-// ---------------------------------------------------------------------------
-// Scratch stores.  A warp stages the 32 rows x 32 columns it read from tensor memory in a buffer of its own
-// (128-byte rows, the 128-byte swizzle that the tensor map expects) and its first lane stores them with TMA; no
-// other warp is waited for.  With one 128-row store for four warps, two barriers per 32 columns made the
-// epilogue of a 128 x 256 tile 12 thousand cycles long -- longer than its products at K = 512 (8 thousand).
-// two_buffers: the caller alternates between two buffers, so one earlier store may still be reading.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void stage_and_store(const CUtensorMap *tmY, uint8_t *buf, const uint32_t (&r)[32], int lane,
-                                                int x, int y, int rows_valid, bool two_buffers) {
-    if (lane == 0) {
-        if (two_buffers) bulk_wait_read_1();
-        else bulk_wait_read_0();
-    }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        *reinterpret_cast<uint4 *>(buf + lane * 128 + ((j ^ (lane & 7)) * 16)) =
-            make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
-    fence_proxy_async_smem();
-    __syncwarp();
-    if (lane == 0 && y < rows_valid) {
-        tma_store_2d(tmY, buf, x, y);
-        bulk_commit();
-    }
 }
 
 // ---------------------------------------------------------------------------

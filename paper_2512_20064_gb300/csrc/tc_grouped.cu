@@ -73,8 +73,9 @@ constexpr int kTaskRing = 16;
 constexpr int kPBarrierBytes = 3072;
 constexpr int kMeasureParts = 4;                   // measurements of an m-tile: 32 rows each
 constexpr int kMeasureGroups = 2;                  // groups of four warps per block
-constexpr int kMeasureSums = 1024;                 // (row, outcome) sums of a group in shared memory
+constexpr int kMeasureSums = 896;                  // (row, outcome) sums of a group in shared memory
 constexpr int kPMeasureBytes = kMeasureGroups * kMeasureSums * 8;
+constexpr int kPStageBytes = 4 * kYWarpBytes;      // scratch staging, one buffer per epilogue warp
 
 struct PParams {
     const PSegment *segs;
@@ -158,7 +159,8 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     uint8_t *smem = smem_raw + ((1024u - (raw_addr & 1023u)) & 1023u);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + (size_t)p.stages * p.stage_bytes);
+    uint8_t *ystage = smem + (size_t)p.stages * p.stage_bytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(ystage + kPStageBytes);
     uint64_t *empty = full + p.stages;
     uint64_t *tfull = empty + p.stages;
     uint64_t *tempty = tfull + 2;
@@ -365,30 +367,38 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
             tc_fence_after();
             const int row = mt * kBM + quad * 32 + lane;
             const bool valid = row < sg->rows_valid;
-            float *yrow = sg->Y + (int64_t)row * sg->ldY + (int64_t)nt * sg->bn;
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)buf * kAccStride;
             float ss = 0.f;
-            for (int ch = 0; ch < sg->bn / 32; ++ch) {
-                uint32_t r[32];
-                tmem_ld_32x32b_x32(taddr + (uint32_t)(ch * 32), r);
-                tc_wait_ld();
+            const int nch = sg->bn / 32, x0 = nt * sg->bn, y0 = mt * kBM + quad * 32, rows_valid = sg->rows_valid;
+            uint8_t *stage = ystage + (uint32_t)quad * kYWarpBytes;
+            auto put_chunk = [&](const uint32_t (&r)[32], int ch) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
                     const float v = __uint_as_float(r[j]);
                     ss = fmaf(v, v, ss);
                 }
-                if (valid) {
-                    float4 *dst = reinterpret_cast<float4 *>(yrow + ch * 32);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        dst[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
-                                             __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
-                }
+                stage_and_store(&sg->tmY, stage, r, lane, x0 + ch * 32, y0, rows_valid, false);
+            };
+            // the next 32 columns are on their way from tensor memory while a chunk is squared and staged
+            uint32_t ra[32], rb[32];
+            tmem_ld_32x32b_x32(taddr, ra);
+            tc_wait_ld_for(ra);
+            for (int ch = 0; ch < nch; ch += 2) {
+                const bool two = ch + 1 < nch, more = ch + 2 < nch;
+                if (two) tmem_ld_32x32b_x32(taddr + (uint32_t)((ch + 1) * 32), rb);
+                put_chunk(ra, ch);
+                if (!two) break;
+                tc_wait_ld_for(rb);
+                if (more) tmem_ld_32x32b_x32(taddr + (uint32_t)((ch + 2) * 32), ra);
+                put_chunk(rb, ch + 1);
+                if (more) tc_wait_ld_for(ra);
             }
             tc_fence_before();
             mbar_arrive(&tempty[buf]);
             if (valid) sg->P[(int64_t)row * sg->ldP + nt] = ss;
-            // count the tile; the m-tile's last tile puts it on the measurement list
+            // count the tile once its scratch stores are complete; the m-tile's last tile puts it on the
+            // measurement list
+            if (lane == 0) bulk_wait_all();
             named_bar_sync(1, 128);
             if (threadIdx.x == 64) {
                 __threadfence();  // the group's stores (ordered by the barrier) before the count
@@ -500,13 +510,13 @@ cudaError_t launch_batch_persistent(const PersistentArgs &g, int num_sms, int *d
     for (int q = 0; q < g.nprod; ++q)
         p.prod_code |= ((uint32_t)g.prod_a[q] | ((uint32_t)g.prod_b[q] << 2)) << (4 * q);
     p.stage_bytes = (uint32_t)g.a_planes * kATileBytes + (uint32_t)g.b_planes * kBPlaneBytesMax;
-    p.stages = (kSmemLimit - 1024 - kPBarrierBytes - kPMeasureBytes) / (int)p.stage_bytes;
+    p.stages = (kSmemLimit - 1024 - kPBarrierBytes - kPMeasureBytes - kPStageBytes) / (int)p.stage_bytes;
     if (p.stages > kMaxStages) p.stages = kMaxStages;
     if (p.stages < 2) return cudaErrorInvalidConfiguration;
     p.limit_ns = g.wait_limit_ns;
     p.stall = g.stall_test ? 1 : 0;
     p.err = d_err;
-    const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + kPBarrierBytes + kPMeasureBytes;
+    const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + kPBarrierBytes + kPMeasureBytes + kPStageBytes;
     const int grid = g.total_tasks < num_sms ? (int)g.total_tasks : num_sms;
     tc_batch_persistent_kernel<<<grid, kPThreads, smem, st>>>(p);
     return cudaGetLastError();
