@@ -19,6 +19,12 @@
 // Two accumulator buffers of 256 columns let the epilogue of tile i overlap
 // the main loop of tile i+1.
 //
+// Pair variant (kPair; two-pass and promoted): a cluster of two CTAs computes 256 rows x bn columns with
+// tcgen05 cta_group::2.  Each CTA loads its own 128 rows and half of the columns and drains its own 128 rows;
+// both CTAs' copies complete on the barriers of CTA 0, whose MMA thread issues the M = 256 products and commits
+// to both.  A CTA takes in 48 KB per k-block instead of 64 (two left planes, one site plane, bn = 256), near the
+// most an SM can (64 bytes a cycle), and holds one more pipeline stage.
+//
 // Fused variant (320 threads): warps 6-9 measure.  Each thread block owns
 // whole m-tiles (128 rows) and walks all their n-tiles in order; after the
 // last n-tile of an m-tile the epilogue hands it to the block's measurement
@@ -93,7 +99,7 @@ struct TcParams {
     int num_m_tiles, num_n_tiles, num_k_blocks, bn;
     int a_planes, b_planes, stages, nprod;
     uint32_t prod_code;  // product q uses A plane (code >> 4q) & 3 and B plane (code >> (4q+2)) & 3
-    int tma_store;       // epilogue stages 128 x 32 chunks in shared memory and stores them with TMA
+    int tma_store;       // epilogue stages 32 x 32 chunks in shared memory and stores them with TMA
     uint32_t stage_bytes, b_plane_bytes;
     int row0;
     uint32_t idesc;
@@ -956,7 +962,10 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
 }
 
 // Whether a launch runs on CTA pairs (see kPair): if its units of two m-tiles and one n-tile, one per pair, take no
-// more rounds than its tiles, one per CTA -- an odd last m-tile leaves half a pair idle.
+// more rounds than its tiles, one per CTA -- an odd last m-tile leaves half a pair idle.  Measured, singles / pairs:
+// FP16x3, 5003 rows, K = 1600, 33 sites 4.80 / 4.27 ms (a third stage fits); BF16x2, 8192 rows, K = 4032, 24 sites
+// 13.8 / 13.2; 131072 rows, K = 512, 128 sites 60.0 / 58.0; 256 rows, K = 1024, 20 sites (with loads) 4.23 / 4.01.
+// Tiles narrower than 128 columns stay with single CTAs: half of such a tile is a copy of a few KB.
 bool pair_pays(const TcArgs &a, const TcParams &p, int num_sms) {
     if (!a.has_pair || a.fp8 || p.bn < 128 || p.num_m_tiles < 2) return false;
     const int64_t pairs = num_sms / 2, units = (int64_t)((p.num_m_tiles + 1) / 2) * p.num_n_tiles;
