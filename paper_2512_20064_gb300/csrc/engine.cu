@@ -89,11 +89,11 @@ struct ChainPlan {
 // Both sides in microseconds, fitted to measurements (24-site chains, 1 to 131072 rows, d = 2..6, chi = 8..256):
 //   one launch:  per wave of blocks (three per SM, fewer where shared memory says so) and site 3.6, plus 0.67
 //                for each stage of 16 K-entries x 128 columns;
-//   two launches: 22 per site (two launches, an event each way), plus the products at 52 TFLOP/s on whole
+//   two launches: 18 per site (two launches and their timing events), plus the products at 52 TFLOP/s on whole
 //                64-column halves, the scratch, selected and next rows at 5 TB/s, and the FP64 draws.
-// E.g. d = 2, chi = 32: 64 rows 151 against 584 us, 131072 rows 1731 against 2407; d = 4, chi = 64: 4864 rows
-// 645 against 866, 10000 rows 1852 against 1376 (two launches); chi = 128 and up: two launches.  Where the two
-// estimates are close the two-launch path stays (the factor 0.8: d = 6, chi = 90, 4864 rows 2160 against 1800).
+// E.g. d = 2, chi = 32: 64 rows 152 against 474 us, 131072 rows 1732 against 2534; d = 4, chi = 64: 4864 rows
+// 645 against 756, but 2048 rows 645 against 616 and 10000 rows 1854 against 1253 (two launches); chi = 128 and
+// up: two launches.  Where the two estimates are close the two-launch path stays (the factor 0.9).
 bool chain_plan(const std::vector<Tensor *> &ts, int d, int64_t N, int num_sms, ChainPlan *c) {
     c->sites.clear();
     double one = 0.0, two = 0.0;  // one: per wave of blocks
@@ -110,14 +110,14 @@ bool chain_plan(const std::vector<Tensor *> &ts, int d, int64_t N, int num_sms, 
         c->p_ld = std::max(c->p_ld, d * s.tiles_per_s);
         if (c->k_max > 1024 || c->y_ld > 2048) return false;  // wider than a block's shared memory
         one += 3.6 + 0.67 * (s.K / 16) * std::ceil(d * (double)roundup(s.nreal, 16) / 128.0);
-        two += 22.0 + (double)N * (1.9e-4 + (double)t->L.K_pad * d * (double)roundup(s.nreal, 64) / 26e6 +
+        two += 18.0 + (double)N * (1.9e-4 + (double)t->L.K_pad * d * (double)roundup(s.nreal, 64) / 26e6 +
                                    4.0 * ((d + 2.0) * s.nreal + s.nreal) / 5e6);
     }
     const size_t smem = chain_f32_smem(c->k_max, c->y_ld, c->p_ld, d);
     if (smem > kChainSmemLimit) return false;
     const int64_t per_sm = std::min<int64_t>(kChainBlocksPerSm, (int64_t)(kChainSmemLimit / (smem + 1024)));
     const int64_t slots = std::max<int64_t>(1, per_sm) * num_sms;
-    return (double)((chain_f32_blocks(N) + slots - 1) / slots) * one < 0.8 * two;
+    return (double)((chain_f32_blocks(N) + slots - 1) / slots) * one < 0.9 * two;
 }
 
 }  // namespace
