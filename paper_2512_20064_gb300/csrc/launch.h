@@ -219,7 +219,7 @@ struct PSegment {  // 64-byte aligned through its CUtensorMap members
     uint32_t idesc, tx_bytes;
     int row0;            // TMA y coordinate of the chunk's first row in the job's left-operand buffers
     int step;            // c * M + k: steps every m-tile of this chunk has been measured for before this segment
-    int64_t slot_base;   // measured[slot_base + mt]: 32-row measurements completed by m-tile slot mt of the job
+    int64_t slot_base;   // measured[slot_base + mt]: measurements completed by m-tile slot mt of the job (`parts` per step)
     int64_t done_base;   // tiles_done[done_base + mt]: finished tiles of m-tile mt of this segment
     float *P;
     int ldP;
@@ -232,6 +232,7 @@ struct PersistentArgs {
     int nseg;
     int64_t total_tasks;
     int64_t total_m_tiles;     // of all segments
+    int parts;                 // measurements of an m-tile, 128 / parts rows each: 4, 8 or 16
     int *queue;                // device: next task, 64 bits (zero at launch)
     int *measure_queue;        // device: next measurement, 64 bits (zero at launch)
     int *ready_tail;           // device: m-tiles put on the measurement list (zero at launch)

@@ -57,10 +57,10 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity) 
 // epilogue stores the FP32 tile and its sums of squares and counts the finished
 // tiles of the m-tile; the thread that counts the last one publishes the m-tile
 // in the launch's measurement list.  Measurements are handed out like tasks: each
-// group of four measurement warps takes the next 32 rows of the list from a global
+// group of four measurement warps takes the next 128 / parts rows of the list from a global
 // counter, in the order of publication, waits (bounded) for them to be published,
 // draws, writes the next left rows (Algorithm 2) and adds one to the slot's counter,
-// which stands at kMeasureParts for every step measured.  Warps: 0 TMA producer,
+// `parts` for every step measured.  Warps: 0 TMA producer,
 // 1 MMA issuer, 2-5 epilogue, 6-13 two measurement groups (448 threads).
 //
 // The list is what keeps a step short: the steps of a chain follow each other, and
@@ -71,7 +71,7 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity) 
 constexpr int kPThreads = 448;
 constexpr int kTaskRing = 16;
 constexpr int kPBarrierBytes = 3072;
-constexpr int kMeasureParts = 4;                   // measurements of an m-tile: 32 rows each
+constexpr int kMeasureRows = 32;                   // most rows of one measurement
 constexpr int kMeasureGroups = 2;                  // groups of four warps per block
 constexpr int kMeasureSums = 896;                  // (row, outcome) sums of a group in shared memory
 constexpr int kPMeasureBytes = kMeasureGroups * kMeasureSums * 8;
@@ -88,6 +88,7 @@ struct PParams {
     int *ready_tail;            // entries published
     unsigned long long *measure_queue;  // next 32-row measurement
     int64_t total_measures;
+    int parts;                  // measurements of an m-tile: 128 / parts rows each
     int stages, a_planes, b_planes, nprod;
     uint32_t prod_code, stage_bytes;
     uint64_t limit_ns;
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
                 const int64_t lt = t - sg->task_begin;
                 const int mt = (int)(lt / sg->num_n_tiles);
                 const int nt = (int)(lt - (int64_t)mt * sg->num_n_tiles);
-                const int target = (sg->step + p.stall) * kMeasureParts;
+                const int target = (sg->step + p.stall) * p.parts;
                 if (target > 0) {
                     bool timed_out;
                     if (!wait_counter(p.measured + sg->slot_base + mt, target, p, &timed_out)) {
@@ -425,10 +426,10 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
                 if (q < p.total_measures) {
                     unsigned long long e = 0;
                     bool timed_out;
-                    if (wait_entry(p.ready + q / kMeasureParts, p, &e, &timed_out)) {
+                    if (wait_entry(p.ready + q / p.parts, p, &e, &timed_out)) {
                         si = (int)(e >> 32) - 1;
                         now[1] = (int)(unsigned)e;
-                        now[2] = (int)(q % kMeasureParts);
+                        now[2] = (int)(q % p.parts);
                     } else if (timed_out) {
                         record_error(p.err, abort_flag, kDevTimeoutMeasure);
                     }
@@ -440,10 +441,11 @@ __global__ void __launch_bounds__(kPThreads, 1) tc_batch_persistent_kernel(const
             if (si < 0) break;
             const int mt = now[1];
             const MeasureArgs &a = p.meas[si];
-            const int r0 = mt * kBM + now[2] * (kBM / kMeasureParts);
-            const int count = min(kBM / kMeasureParts, p.segs[si].rows_valid - r0);
+            const int part_rows = kBM / p.parts;
+            const int r0 = mt * kBM + now[2] * part_rows;
+            const int count = min(part_rows, p.segs[si].rows_valid - r0);
             const int d = a.d, T = a.tiles_per_s;
-            const bool in_smem = d * (kBM / kMeasureParts) <= kMeasureSums;
+            const bool in_smem = d * part_rows <= kMeasureSums;
             if (in_smem) {
                 for (int e = m; e < count * d; e += 128) {
                     const int r = e / d;
@@ -488,6 +490,7 @@ cudaError_t prepare_batch_persistent() {
 
 cudaError_t launch_batch_persistent(const PersistentArgs &g, int num_sms, int *d_err, cudaStream_t st) {
     if (g.nseg <= 0 || g.total_tasks <= 0) return cudaSuccess;
+    if (g.parts < kBM / kMeasureRows || kBM % g.parts != 0) return cudaErrorInvalidValue;
     if (g.nprod < 1 || g.nprod > kMaxProducts || g.a_planes < 1 || g.a_planes > 3 || g.b_planes < 1 ||
         g.b_planes > 2)
         return cudaErrorInvalidValue;
@@ -502,7 +505,8 @@ cudaError_t launch_batch_persistent(const PersistentArgs &g, int num_sms, int *d
     p.ready = reinterpret_cast<unsigned long long *>(g.ready);
     p.ready_tail = g.ready_tail;
     p.measure_queue = reinterpret_cast<unsigned long long *>(g.measure_queue);
-    p.total_measures = g.total_m_tiles * kMeasureParts;
+    p.parts = g.parts;
+    p.total_measures = g.total_m_tiles * g.parts;
     p.a_planes = g.a_planes;
     p.b_planes = g.b_planes;
     p.nprod = g.nprod;
