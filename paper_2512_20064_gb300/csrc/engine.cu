@@ -4,7 +4,8 @@
 // of the left operand stay resident in device memory (the macro-batch);
 // for each site k the rows are processed in micro-batches: one contraction
 // launch writes the FP32 scratch Y and per-tile sums of squares, one
-// measurement launch draws the outcome and writes the next left operand.  In
+// measurement launch draws the outcome and writes the next left operand.  FP32
+// calls of narrow chains or few rows run in one launch instead (chain_plan).  In
 // host-streaming residency the BF16 site tensor of site k+1 is copied from
 // pinned host memory into one of two device slots on a copy stream while site
 // k computes (Sec. 3.1 double buffer; Sec. 3.3.2 16-bit storage).
