@@ -415,7 +415,10 @@ constexpr uint32_t kYWarpBytes = 4096;  // a warp's 32 x 32 FP32 chunk of the sc
 // (128-byte rows, the 128-byte swizzle that the tensor map expects) and its first lane stores them with TMA; no
 // other warp is waited for.  With one 128-row store for four warps, two barriers per 32 columns made the
 // epilogue of a 128 x 256 tile 12 thousand cycles long -- longer than its products at K = 512 (8 thousand).
-// two_buffers: the caller alternates between two buffers, so one earlier store may still be reading.
+// two_buffers: the caller alternates between two buffers, so one earlier store may still be reading.  Every chunk
+// commits a group, also one past the valid rows, which stores nothing: "at most one group still reading" then means
+// that the group of the chunk before last, the last one to use this buffer, is done.  Were only stores counted, the
+// second chunk past the rows would pass the wait with the last store's buffer still being read, and overwrite it.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void stage_and_store(const CUtensorMap *tmY, uint8_t *buf, const uint32_t (&r)[32], int lane,
                                                 int x, int y, int rows_valid, bool two_buffers) {
@@ -430,8 +433,8 @@ __device__ __forceinline__ void stage_and_store(const CUtensorMap *tmY, uint8_t 
             make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
     fence_proxy_async_smem();
     __syncwarp();
-    if (lane == 0 && y < rows_valid) {
-        tma_store_2d(tmY, buf, x, y);
+    if (lane == 0) {
+        if (y < rows_valid) tma_store_2d(tmY, buf, x, y);
         bulk_commit();
     }
 }
