@@ -706,6 +706,14 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
                     for (int s = 0; s < p.stages; ++s)
                         if (last_parity[s] >= 0) mbar_wait_drain(&full[s], (uint32_t)last_parity[s]);
                 }
+            } else if (kPair) {
+                // the leader's commits arrive on the barriers of both CTAs: the last one on every stage has to be
+                // here before this CTA may leave (nothing orders it before the arrival that the epilogue waits for)
+                for (int s = 0; s < p.stages; ++s)
+                    if (last_parity[s] >= 0 && !mbar_wait_bounded(&empty[s], (uint32_t)last_parity[s], abort_flag)) {
+                        record_error(p.err, abort_flag, kDevTimeoutProducer);
+                        break;
+                    }
             }
         }
         __syncwarp();
