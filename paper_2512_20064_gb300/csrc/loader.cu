@@ -196,6 +196,12 @@ static bool operands_fit(const Tensor &from, int precision, const SiteLayout &L)
     return fits(from.B_hi) && (plan_of(precision).b_planes < 2 || fits(from.B_lo));
 }
 
+// Test hook: FASTMPS_TEST_FAIL_TENSOR_MAPS=1 makes a load report that the maps over its operands could not be encoded.
+static bool map_failure_requested() {
+    const char *v = getenv("FASTMPS_TEST_FAIL_TENSOR_MAPS");
+    return v && v[0] == '1';
+}
+
 static int load_resident(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const void *src, int dtype,
                          const void *lam_dev);
 
@@ -291,13 +297,15 @@ int load_tensor(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const 
     return rc;
 }
 
-// Repack of the tensor at src (device) into t's operands.
+// Repack of the tensor at src (device) into t's operands.  Whatever can fail comes before the first kernel that writes
+// them: they may be those of the site that t replaces, which stays if the load is refused.
 static int load_resident(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_r, const void *src, int dtype,
                          const void *lam_dev) {
     const bool is_f64 = dtype == FASTMPS_C128;
     const int64_t nelem = (int64_t)chi_l * d * chi_r;
     const bool tune = h->opt.autotune && is_bf16(h) && !is_fp8(h) && !is_f16(h) && h->opt.accum_chunk == 0;
-    cudaError_t e;
+    cudaError_t e = cudaGetLastError();  // an error left by an earlier call
+    if (e != cudaSuccess) return cuda_fail(h, e, "repack");
     const size_t op_elems = (size_t)t.L.ncols * t.L.K_pad;
     if (is_fp8(h)) {
         // per-site power-of-two scale that puts the largest |Re|, |Im| in [224, 448]
@@ -317,10 +325,7 @@ static int load_resident(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_
         const bool two = plan_of(h->opt.precision).b_planes > 1;
         if (!t.B_hi.ensure(op_elems * 2) || (two && !t.B_lo.ensure(op_elems * 2)) || !h->err.ensure(256))
             return fail(h, FASTMPS_ERR_OOM, "allocation failed");
-        launch_absmax(src, is_f64, nelem, chi_r, lam_dev, h->err.as<float>(), h->stream);
-        launch_repack_f16(src, is_f64, lam_dev, h->err.as<float>(), t.L, t.B_hi.as<uint16_t>(),
-                          two ? t.B_lo.as<uint16_t>() : nullptr, h->stream);
-        if (!encode_2d_f16(&t.tmB[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn) ||
+        if (map_failure_requested() || !encode_2d_f16(&t.tmB[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn) ||
             (two && !encode_2d_f16(&t.tmB[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn)) ||
             !encode_2d_f16(&t.tmBh[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn / 2) ||
             (two && !encode_2d_f16(&t.tmBh[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn / 2)))
@@ -329,6 +334,11 @@ static int load_resident(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_
             t.tmB[1] = t.tmB[0];
             t.tmBh[1] = t.tmBh[0];
         }
+        launch_absmax(src, is_f64, nelem, chi_r, lam_dev, h->err.as<float>(), h->stream);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(h, e, "site tensor maximum");
+        launch_repack_f16(src, is_f64, lam_dev, h->err.as<float>(), t.L, t.B_hi.as<uint16_t>(),
+                          two ? t.B_lo.as<uint16_t>() : nullptr, h->stream);
     } else if (is_bf16(h)) {
         if (tune) {
             std::lock_guard<std::mutex> lock(g_tune_mutex);
@@ -353,8 +363,7 @@ static int load_resident(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_
             if (!t.B_lo.ensure(op_elems * 2)) return fail(h, FASTMPS_ERR_OOM, "site operand allocation failed");
             lo = t.B_lo.as<__nv_bfloat16>();
         }
-        launch_repack_bf16(src, is_f64, lam_dev, t.L, t.B_hi.as<__nv_bfloat16>(), lo, h->stream);
-        if (!encode_2d_bf16(&t.tmB[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn))
+        if (map_failure_requested() || !encode_2d_bf16(&t.tmB[0], t.B_hi.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn))
             return fail(h, FASTMPS_ERR_CUDA, "tensor map encoding failed");
         if (lo && !encode_2d_bf16(&t.tmB[1], t.B_lo.p, t.L.K_pad, t.L.ncols, t.L.K_pad, 64, t.L.bn))
             return fail(h, FASTMPS_ERR_CUDA, "tensor map encoding failed");
@@ -365,6 +374,7 @@ static int load_resident(fastmps_handle h, Tensor &t, int chi_l, int d, int chi_
             t.tmB[1] = t.tmB[0];
             t.tmBh[1] = t.tmBh[0];
         }
+        launch_repack_bf16(src, is_f64, lam_dev, t.L, t.B_hi.as<__nv_bfloat16>(), lo, h->stream);
     } else {
         if (!t.Bt.ensure(op_elems * 4)) return fail(h, FASTMPS_ERR_OOM, "site operand allocation failed");
         launch_repack_f32(h->staging.p, dtype == FASTMPS_C128, t.L, t.Bt.as<float>(), h->stream);

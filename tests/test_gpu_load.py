@@ -73,3 +73,22 @@ def test_reload_over_other_shapes(precision):
                 fresh.load_chain(tt)
                 want = fresh.sample(bb, 3, 150, 3)
             assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("precision", ["bf16x3", "fp16x2"])
+def test_reload_that_fails_late_keeps_the_old_site(precision, monkeypatch):
+    """A load that fails after its operands were chosen (here: their tensor maps) leaves the loaded values alone,
+    although a reload may take over the operands of the site that it replaces."""
+    import paper_2512_20064_gb300 as F
+
+    b, ts = _chain(np.complex64)
+    with F.Sampler(precision=precision) as s:
+        s.load_chain(ts)
+        want = s.sample(b, 3, 150, 3)
+        for k in (4, 6):
+            monkeypatch.setenv("FASTMPS_TEST_FAIL_TENSOR_MAPS", "1")
+            with pytest.raises(F.FastMPSError):
+                s.load_site(k, np.ascontiguousarray(ts[k][:, ::-1, :]))
+            monkeypatch.delenv("FASTMPS_TEST_FAIL_TENSOR_MAPS")
+            got = s.sample(b, 3, 150, 3)
+            assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
