@@ -19,10 +19,13 @@ namespace {
 // candidate: with one thread block per SM the deepest ring that fits shared
 // memory never loses.  Results are cached per process and, when
 // FASTMPS_TUNE_CACHE names a file, in that file as a flat JSON object
-// {"precision:chi_l:d:chi_r": bn + 10000 * mode, ...} (mode 2: cluster).
+// {"version": v, "precision:chi_l:d:chi_r": bn + 10000 * mode, ...} (mode 2:
+// cluster).  The version counts the kernels that the choices were timed on: a
+// file of another one, or of none, is not read and is written anew.
 // ---------------------------------------------------------------------------
 std::mutex g_tune_mutex;
 std::map<std::string, int> g_tuned;
+constexpr int kTuneVersion = 2;  // 2: the two-pass contraction runs on CTA pairs
 bool g_tune_loaded = false;
 
 std::string tune_key(int precision, int chi_l, int d, int chi_r) {
@@ -51,6 +54,9 @@ void tune_cache_load() {
         g_tuned[text.substr(i + 1, j - i - 1)] = atoi(text.c_str() + c + 1);
         i = j + 1;
     }
+    auto version = g_tuned.find("version");
+    if (version == g_tuned.end() || version->second != kTuneVersion) g_tuned.clear();
+    else g_tuned.erase(version);
 }
 
 void tune_cache_store() {
@@ -58,12 +64,8 @@ void tune_cache_store() {
     if (!path) return;
     FILE *f = fopen(path, "w");
     if (!f) return;
-    fputc('{', f);
-    bool first = true;
-    for (auto &kv : g_tuned) {
-        fprintf(f, "%s\"%s\": %d", first ? "" : ", ", kv.first.c_str(), kv.second);
-        first = false;
-    }
+    fprintf(f, "{\"version\": %d", kTuneVersion);
+    for (auto &kv : g_tuned) fprintf(f, ", \"%s\": %d", kv.first.c_str(), kv.second);
     fputs("}\n", f);
     fclose(f);
 }
@@ -112,7 +114,10 @@ int autotune_bn(fastmps_handle h, const void *src, int chi_l, int d, int chi_r, 
             ok = ok && encode_2d_bf16(&ta.tmA[p], V[p < plan.a_planes ? p : 0].p, L.K_pad, rows, L.K_pad, 64, 128);
         for (int p = 0; p < 2; ++p)
             ok = ok && encode_2d_bf16(&ta.tmB[p], B[p < plan.b_planes ? p : 0].p, L.K_pad, L.ncols, L.K_pad, 64, L.bn);
+        for (int p = 0; p < 2; ++p)
+            ok = ok && encode_2d_bf16(&ta.tmBh[p], B[p < plan.b_planes ? p : 0].p, L.K_pad, L.ncols, L.K_pad, 64, L.bn / 2);
         if (!ok) break;
+        ta.has_pair = true;  // as in a call: CTA pairs wherever they pay
         ta.row0 = 0;
         ta.rows_pad = (int)rows;
         ContractOut co{Y.as<float>(), L.ncols, P.as<float>(), L.ncols / L.bn, (int)rows};

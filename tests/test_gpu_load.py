@@ -92,3 +92,29 @@ def test_reload_that_fails_late_keeps_the_old_site(precision, monkeypatch):
             monkeypatch.delenv("FASTMPS_TEST_FAIL_TENSOR_MAPS")
             got = s.sample(b, 3, 150, 3)
             assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+
+
+def test_tune_cache_of_other_kernels_is_not_read(tmp_path):
+    """A choice file without the present version is measured anew (its width of 96 is no candidate); one with it is
+    read and stays as it is."""
+    import json
+    import os
+    import subprocess
+    import sys
+
+    cache = tmp_path / "tune.json"
+    cache.write_text(json.dumps({"1:40:3:40": 96}))
+    code = ("import sys; sys.path.insert(0, %r)\n"
+            "import numpy as np, gen, paper_2512_20064_gb300 as F\n"
+            "b, ts, _ = gen.mps_tensors(9, 3, 40, base_seed=4, skew=1.5, dtype=np.complex64)\n"
+            "with F.Sampler(precision='bf16x2', autotune=True) as s:\n"
+            "    s.load_chain(ts)\n"
+            "    assert np.isfinite(s.sample(b, 3, 300, 1)[1]).all()\n") % os.path.dirname(os.path.dirname(__file__))
+    texts = []
+    for _ in range(2):
+        subprocess.run([sys.executable, "-c", code], env=dict(os.environ, FASTMPS_TUNE_CACHE=str(cache)), check=True,
+                       timeout=300)
+        texts.append(cache.read_text())
+    table = json.loads(texts[0])
+    assert table["1:40:3:40"] == 64 and "version" in table  # 64 columns: the only candidate not wider than the block
+    assert texts[0] == texts[1]
