@@ -182,8 +182,6 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
     if (N == 0) return FASTMPS_OK;
     const bool stream_mode = h->opt.residency == FASTMPS_HOST_STREAM;
     const bool bf16 = is_bf16(h);
-    ChainPlan chain;
-    const bool in_one_launch = !bf16 && !mu_dev && chain_plan(ts, d, N, h->num_sms, &chain);
     cudaStream_t st = h->stream;
     cudaError_t e;
 
@@ -207,6 +205,10 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
     }
     N2 = std::min(N2, N_pad);
     const int64_t J = (N + N2 - 1) / N2;  // micro-batches per site
+    // a caller that bounds the rows of a launch below the call's gets launches of that many rows
+    ChainPlan chain;
+    const bool in_one_launch =
+        !bf16 && !mu_dev && (h->opt.max_microbatch == 0 || J == 1) && chain_plan(ts, d, N, h->num_sms, &chain);
 
     // ---- buffers -------------------------------------------------------------
     const bool fp8 = is_fp8(h);

@@ -61,3 +61,26 @@ def test_one_launch_reports_a_zero_norm():
         assert e.value.code == -8
         s.load_site(3, ts[3])
         assert np.isfinite(s.sample(b, 2, 40, 1)[1]).all()
+
+
+@pytest.mark.parametrize("M,d,chi,one", [(10, 3, 16, True), (10, 2, 40, True), (13, 3, 350, False)])
+def test_micro_batches_of_fp32_calls(M, d, chi, one):
+    """max_microbatch bounds the rows of a launch, so a narrow chain runs in one launch only where all rows fit it (rows
+    of d * 2 chi > 2048 columns never do).  Bit for bit the same for one launch, one micro-batch per site (one stream)
+    and several (two streams)."""
+    import paper_2512_20064_gb300 as F
+
+    N = 1000
+    b, ts, _ = gen.mps_tensors(M, d, chi, base_seed=44, skew=1.5, dtype=np.complex64)
+    out = {}
+    for mb in (0, 256, 1024):
+        with F.Sampler(precision="fp32", max_microbatch=mb) as s:
+            s.load_chain(ts)
+            out[mb] = s.sample(b, d, N, 7, trace_rows=N)
+            st = s.stats()
+            if mb == 256:
+                assert st["contract_launches"] == 4 * M
+            else:
+                assert st["contract_launches"] == (1 if one else M)
+    for mb in (256, 1024):
+        assert all(np.array_equal(x, y) for x, y in zip(out[0], out[mb])), mb
