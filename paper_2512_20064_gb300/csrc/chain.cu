@@ -75,14 +75,14 @@ struct Units {
     int count;  // units of the site
 };
 
-__device__ __forceinline__ Units units_of(const ChainSite &s, int d) {
+__host__ __device__ inline Units units_of(const ChainSite &s, int d) {
     Units u;
     u.Wb = s.nreal > 64 ? 0 : s.nreal > 32 ? 64 : s.nreal > 16 ? 32 : 16;
     u.count = u.Wb ? (d * u.Wb + 127) / 128 : d * s.tiles_per_s;
     return u;
 }
 // Whether columns 64 .. 127 of unit j hold anything.
-__device__ __forceinline__ bool unit_is_wide(const ChainSite &s, const Units &u, int d, int j) {
+__host__ __device__ inline bool unit_is_wide(const ChainSite &s, const Units &u, int d, int j) {
     return u.Wb ? d * u.Wb - j * 128 > 64 : s.nreal - (j % s.tiles_per_s) * 128 > 64;
 }
 
@@ -331,6 +331,13 @@ __global__ void __launch_bounds__(kThreads, kChainBlocksPerSm) chain_f32_kernel(
 }
 
 }  // namespace
+
+void chain_f32_units(const ChainSite &s, int d, int *wide, int *narrow) {
+    const Units u = units_of(s, d);
+    *wide = 0;
+    for (int j = 0; j < u.count; ++j) *wide += unit_is_wide(s, u, d, j) ? 1 : 0;
+    *narrow = u.count - *wide;
+}
 
 int64_t chain_f32_blocks(int64_t rows) { return (rows + kRows - 1) / kRows; }
 

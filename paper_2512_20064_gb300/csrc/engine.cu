@@ -86,18 +86,20 @@ struct ChainPlan {
     int k_max = 0, y_ld = 0, p_ld = 0;
 };
 
-// Whether an FP32 call runs in one launch: if its estimated time is well below that of two launches per site.
-// Both sides in microseconds, fitted to measurements (24-site chains, 1 to 131072 rows, d = 2..6, chi = 8..256):
-//   one launch:  per wave of blocks (three per SM, fewer where shared memory says so) and site 3.6, plus 0.67
-//                for each stage of 16 K-entries x 128 columns;
-//   two launches: 18 per site (two launches and their timing events), plus the products at 52 TFLOP/s on whole
-//                64-column halves, the scratch, selected and next rows at 5 TB/s, and the FP64 draws.
-// E.g. d = 2, chi = 32: 64 rows 152 against 474 us, 131072 rows 1732 against 2534; d = 4, chi = 64: 4864 rows
-// 645 against 756, but 2048 rows 645 against 616 and 10000 rows 1854 against 1253 (two launches); chi = 128 and
-// up: two launches.  Where the two estimates are close the two-launch path stays (the factor 0.9).
+// Whether an FP32 call runs in one launch: if its estimated time is below that of two launches per site.  Both
+// sides in microseconds, fitted to 216 measured calls (24-site chains, 1 to 131072 rows, d = 2..10, chi = 5..160, odd
+// widths among them).  Over these and 72 others the chosen side takes 1.005 of the better one's time on average, 1.06
+// at worst where it was fitted, 1.21 elsewhere (d = 4, chi = 40, 10000 rows: 1.27 ms for 1.05):
+//   one launch:  per wave of blocks 2.6 a site, plus 0.92 for each unit of 128 columns and 0.59 for each of 64 that
+//                the kernel passes per 16 K-entries (chain_f32_units), 46 % more for every further block on an SM
+//                (at most three, fewer where shared memory says so);
+//   two launches: 15 a site (two launches and their timing events) and 0.049 per K entry (a tile's latency), plus per
+//                row 3.7e-4 (the FP64 draw) and the products at 48 TFLOP/s on whole 64-column halves.
+// E.g. (one / two) d = 2, chi = 32: 64 rows 155 / 477, 131072 rows 1735 / 2521; d = 4, chi = 64: 4864 rows 645 / 747,
+// 64 rows 636 / 561; d = 10, chi = 33: 64 rows 1118 / 580, 10000 rows 3286 / 2199; d = 6, chi = 90 and up: two.
 bool chain_plan(const std::vector<Tensor *> &ts, int d, int64_t N, int num_sms, ChainPlan *c) {
     c->sites.clear();
-    double one = 0.0, two = 0.0;  // one: per wave of blocks
+    double latency = 0.0, units = 0.0, two = 0.0;  // latency, units: of one block
     for (const Tensor *t : ts) {
         ChainSite s;
         s.Bt = t->Bt.as<float>();
@@ -110,15 +112,19 @@ bool chain_plan(const std::vector<Tensor *> &ts, int d, int64_t N, int num_sms, 
         c->y_ld = std::max(c->y_ld, d * (int)roundup(s.nreal, 4));
         c->p_ld = std::max(c->p_ld, d * s.tiles_per_s);
         if (c->k_max > 1024 || c->y_ld > 2048) return false;  // wider than a block's shared memory
-        one += 3.6 + 0.67 * (s.K / 16) * std::ceil(d * (double)roundup(s.nreal, 16) / 128.0);
-        two += 18.0 + (double)N * (1.9e-4 + (double)t->L.K_pad * d * (double)roundup(s.nreal, 64) / 26e6 +
-                                   4.0 * ((d + 2.0) * s.nreal + s.nreal) / 5e6);
+        int wide, narrow;
+        chain_f32_units(s, d, &wide, &narrow);
+        latency += 2.6;
+        units += (s.K / 16) * (0.92 * wide + 0.59 * narrow);
+        two += 15.0 + 0.049 * t->L.K_pad +
+               (double)N * (3.7e-4 + (double)t->L.K_pad * d * (double)roundup(s.nreal, 64) / 24e6);
     }
     const size_t smem = chain_f32_smem(c->k_max, c->y_ld, c->p_ld, d);
     if (smem > kChainSmemLimit) return false;
     const int64_t per_sm = std::min<int64_t>(kChainBlocksPerSm, (int64_t)(kChainSmemLimit / (smem + 1024)));
-    const int64_t slots = std::max<int64_t>(1, per_sm) * num_sms;
-    return (double)((chain_f32_blocks(N) + slots - 1) / slots) * one < 0.9 * two;
+    const int64_t blocks = chain_f32_blocks(N), slots = std::max<int64_t>(1, per_sm) * num_sms;
+    const int64_t waves = (blocks + slots - 1) / slots, resident = std::min((blocks + num_sms - 1) / num_sms, slots / num_sms);
+    return (double)waves * (latency + units * (1.0 + 0.46 * (double)(resident - 1))) < two;
 }
 
 }  // namespace

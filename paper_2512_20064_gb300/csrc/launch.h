@@ -93,6 +93,8 @@ struct ChainArgs {
 constexpr int kChainBlocksPerSm = 3;  // as far as registers go
 size_t chain_f32_smem(int k_max, int y_ld, int p_ld, int d);
 int64_t chain_f32_blocks(int64_t rows);
+// Column units that a block passes for every 16 K-entries of a site: of 128 columns, and of 64.
+void chain_f32_units(const ChainSite &s, int d, int *wide, int *narrow);
 cudaError_t launch_chain_f32(const ChainArgs &a, cudaStream_t st);
 
 // tcgen05 BF16 split-precision contraction.  tmA[p] / tmB[p] are tensor maps

@@ -84,3 +84,20 @@ def test_micro_batches_of_fp32_calls(M, d, chi, one):
                 assert st["contract_launches"] == (1 if one else M)
     for mb in (256, 1024):
         assert all(np.array_equal(x, y) for x, y in zip(out[0], out[mb])), mb
+
+
+@pytest.mark.parametrize("d,chi,N,one", [
+    (10, 33, 10000, False),  # ten tiles, not seven: 3.29 ms in one launch, 2.20 in two a site
+    (10, 33, 131072, False),
+    (2, 64, 131072, False),
+    (3, 16, 10000, True),
+    (2, 32, 64, True),
+])
+def test_narrow_chains_take_the_shorter_route(d, chi, N, one):
+    import paper_2512_20064_gb300 as F
+
+    b, ts, _ = gen.mps_tensors(24, d, chi, base_seed=8, skew=1.5, dtype=np.complex64)
+    with F.Sampler(precision="fp32") as s:
+        s.load_chain(ts)
+        s.sample(b, d, N, 1)
+        assert (s.stats()["contract_launches"] == 1) == one
