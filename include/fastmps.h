@@ -97,7 +97,8 @@ typedef struct fastmps_options {
     int precision;          /* FASTMPS_FP32 | _BF16X2 | _BF16X3 | _BF16X3L | _BF16X4 | _FP8X1 | _FP8X2 | _FP16X2 |
                                _FP16X3 */
     int residency;          /* FASTMPS_RESIDENT_HBM | FASTMPS_HOST_STREAM (BF16 and FP16 modes only) */
-    int64_t max_microbatch; /* rows per contraction launch; 0 = chosen from free memory */
+    int64_t max_microbatch; /* most rows per launch, rounded down to a multiple of 128 (at least 128);
+                               0 = chosen by the library */
     int autotune;           /* 1: time the candidate tile shapes once per new shape */
     void *stream;           /* cudaStream_t to run on; NULL = a stream owned by the handle */
     int fused_measure;      /* BF16 modes: 0 (default) = separate measurement kernel, overlapped
@@ -128,8 +129,15 @@ typedef struct fastmps_ctx *fastmps_handle;
 /* Per-call statistics of the last fastmps_sample* call on a handle. */
 typedef struct fastmps_stats {
     double ms_total;        /* wall time of the call (host clock) */
-    double ms_contract;     /* device time in contraction kernels (CUDA events) */
-    double ms_measure;      /* device time in the measurement kernels */
+    double ms_contract;     /* device time of the contractions (CUDA events).  With one micro-batch per
+                               site each is timed from the end of the kernel before it, so that gaps
+                               between launches are in it.  An FP32 call that runs in one launch
+                               (narrow chains, few rows) has all its device time here: draws and
+                               next rows are part of that kernel. */
+    double ms_measure;      /* device time of the measurement kernels, from the end of their
+                               contraction where a site has one micro-batch (with displacement, a wait
+                               for the rows' matrices, formed beside the contraction, is in it);
+                               0 where the contraction's kernel measures */
     int64_t launches;       /* kernels launched by the call */
     int64_t contract_launches;
     double flops_algorithmic; /* 8 * N * sum_k chi_l d chi_r */

@@ -51,3 +51,9 @@ def test_clock_record_flags_thermal_slowdown_and_tolerates_missing_power():
 def test_clock_record_without_samples_is_none():
     assert _sampler([]).stop() is None
     assert bench.ClockSampler(0).stop() is None
+
+
+def test_fp32_line_names_the_kernel_that_ran():
+    assert bench.f32_kernel(contract_launches=5, steps=5, M=12) == "chain_f32_kernel"
+    assert bench.f32_kernel(contract_launches=60, steps=5, M=12) == "contract_f32_kernel"
+    assert bench.f32_kernel(contract_launches=5, steps=5, M=1) == "contract_f32_kernel"
