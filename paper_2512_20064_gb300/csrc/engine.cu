@@ -214,7 +214,7 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
     // a caller that bounds the rows of a launch below the call's gets launches of that many rows
     ChainPlan chain;
     const bool in_one_launch =
-        !bf16 && !mu_dev && (h->opt.max_microbatch == 0 || J == 1) && chain_plan(ts, d, N, h->num_sms, &chain);
+        !bf16 && !mu_dev && (h->opt.max_microbatch <= 0 || J == 1) && chain_plan(ts, d, N, h->num_sms, &chain);
 
     // ---- buffers -------------------------------------------------------------
     const bool fp8 = is_fp8(h);
