@@ -538,7 +538,7 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
                     e = launch_contract_tc(ta, L, co, h->num_sms, d_err, st, fused ? &ma : nullptr);
                 if (e != cudaSuccess) return cuda_fail(h, e, "contraction launch");
             } else {
-                launch_contract_f32(h->V[cur][0].as<float>(), ldV, r0, t->Bt.as<float>(), L, co, st);
+                launch_contract_f32(h->V[cur][0].as<float>(), ldV, r0, t->Bt.as<float>(), L, co, h->num_sms, st);
             }
             h->stats.launches += 1;
             h->stats.contract_launches += 1;
@@ -554,7 +554,7 @@ int run_sample(fastmps_handle h, int M, int d, const int *bonds, int64_t n0, int
                     cudaEventRecord(m0, ms);
                 }
                 if (ma.mu) launch_measure_displaced(ma, ms);
-                else launch_measure(ma, ms);
+                else launch_measure(ma, h->num_sms, ms);
                 h->stats.launches += 1;
                 cudaEventRecord(m1, ms);
                 if (ma.mu) {

@@ -573,7 +573,7 @@ contract_f32_kernel(const float *__restrict__ V, int64_t ldV, int64_t row0, cons
 }
 
 void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, const float *Bt, const SiteLayout &L,
-                         const ContractOut &o, cudaStream_t st) {
+                         const ContractOut &o, int num_sms, cudaStream_t st) {
     // 128-row tiles, unless 64- or 32-row tiles still fit one per SM: a lone block per SM runs at half the
     // pace of two, and a shorter tile ends sooner.  Measured, us (128 / 64 / 32 rows): d = 4, chi = 256,
     // 64 rows: 66 / 39 / 33; 512 rows: 66 / 39 / 58; 1024 rows: 66 / 68 / 109.  128 rows at most, so that no
@@ -589,8 +589,8 @@ void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, const float 
                                                                     o.ldP, o.rows_valid, L.tiles_per_s, 2 * L.chi_r,
                                                                     (int)num_m);
     };
-    if (nx * ((o.rows_valid + 31) / 32) <= 152) run(std::integral_constant<int, 2>());
-    else if (nx * ((o.rows_valid + 63) / 64) <= 152) run(std::integral_constant<int, 4>());
+    if (nx * ((o.rows_valid + 31) / 32) <= num_sms) run(std::integral_constant<int, 2>());
+    else if (nx * ((o.rows_valid + 63) / 64) <= num_sms) run(std::integral_constant<int, 4>());
     else run(std::integral_constant<int, 8>());
 }
 
@@ -647,14 +647,14 @@ __global__ void __launch_bounds__(MEASURE_THREADS) measure_kernel(const MeasureA
     if (tid < count) measure_finish(a, r0 + tid, ws, Z, ok, lp, w);
 }
 
-void launch_measure(const MeasureArgs &a, cudaStream_t st) {
+void launch_measure(const MeasureArgs &a, int num_sms, cudaStream_t st) {
     if (a.rows <= 0) return;
     // Rows per block: a warp's worth, so that the FP64 draw (a warp-wide FP64 instruction costs the SM 16
     // cycles however many lanes it has) stays a small part; fewer where rows are wide (65536 rows of 2048
     // entries: 204 us with 32 rows per block, 180 with 16) or where that would leave less than four blocks
     // per SM (5003 rows of 1554 entries: 60 us with 32, 24 with 8); at most MEASURE_SUMS sums.
     int R = MEASURE_ROWS;
-    while (R > 4 && (R * a.K_next > 32768 || (a.rows + R - 1) / R < 4 * 152 || R * a.d > MEASURE_SUMS)) R >>= 1;
+    while (R > 4 && (R * a.K_next > 32768 || (a.rows + R - 1) / R < 4 * num_sms || R * a.d > MEASURE_SUMS)) R >>= 1;
     const int grid = (a.rows + R - 1) / R;
     if (a.f16 || a.V8) measure_kernel<true><<<grid, MEASURE_THREADS, 0, st>>>(a, R);
     else measure_kernel<false><<<grid, MEASURE_THREADS, 0, st>>>(a, R);

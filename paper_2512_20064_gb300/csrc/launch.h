@@ -65,8 +65,9 @@ struct ContractOut {
 };
 
 // FP32 SIMT: Y = V[row0 : row0+o.rows_valid] (ld = ldV, K = L.K_pad) x Bt.  V holds a multiple of 128 rows.
+// num_sms (here and in launch_measure): blocks are made smaller where fewer than that would leave SMs idle.
 void launch_contract_f32(const float *V, int64_t ldV, int64_t row0, const float *Bt, const SiteLayout &L,
-                         const ContractOut &o, cudaStream_t st);
+                         const ContractOut &o, int num_sms, cudaStream_t st);
 
 // FP32, a whole chain in one launch (chain.cu).  sites: device table; y_ld >= d * roundup(2 chi_r, 4) and a
 // multiple of 4, p_ld >= d * tiles_per_s, k_max >= K of every site.
@@ -177,7 +178,7 @@ struct MeasureArgs {
     const int *trace_slot = nullptr;  // nullable: per call row, its trace slot (-1: not traced)
     int *err;
 };
-void launch_measure(const MeasureArgs &a, cudaStream_t st);
+void launch_measure(const MeasureArgs &a, int num_sms, cudaStream_t st);
 
 // ---- Vidal form and GBS displacement (gbs.cu) ------------------------------
 constexpr int kMaxDisplacedD = 16;

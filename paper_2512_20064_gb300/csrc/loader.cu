@@ -150,7 +150,7 @@ int autotune_bn(fastmps_handle h, const void *src, int chi_l, int d, int chi_r, 
                 launch_contract_tc_cluster(ta, L, (int)rows, err.as<int>(), h->stream, ma);
             } else {
                 launch_contract_tc(ta, L, co, h->num_sms, err.as<int>(), h->stream);
-                launch_measure(ma, h->stream);
+                launch_measure(ma, h->num_sms, h->stream);
             }
             cudaEventRecord(e1, h->stream);
             cudaEventSynchronize(e1);

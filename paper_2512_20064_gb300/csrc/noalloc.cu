@@ -215,7 +215,7 @@ extern "C" int fastmps_sample_noalloc(fastmps_handle h, int M, int d, const int 
                 e = launch_contract_tc(ta, L, co, hv.num_sms, d_err, st);
                 if (e != cudaSuccess) return set_error(h, FASTMPS_ERR_CUDA, "contraction launch failed");
             } else {
-                launch_contract_f32(V32[cur], ldV, r0, sv.Bt, L, co, st);
+                launch_contract_f32(V32[cur], ldV, r0, sv.Bt, L, co, hv.num_sms, st);
             }
             MeasureArgs ma;
             ma.Y = Y;
@@ -242,7 +242,7 @@ extern "C" int fastmps_sample_noalloc(fastmps_handle h, int M, int d, const int 
             ma.trace = nullptr;
             ma.trace_rows = 0;
             ma.err = d_err;
-            launch_measure(ma, st);
+            launch_measure(ma, hv.num_sms, st);
             e = cudaGetLastError();
             if (e != cudaSuccess) return set_error(h, FASTMPS_ERR_CUDA, "kernel launch failed");
         }
