@@ -1,7 +1,7 @@
 """The stand-alone measurement kernel at the edges of its row groups, row widths and storage formats
-(needs a GB300).  A block takes 4 to 32 rows depending on the row count, rows are written in 16-byte
-pieces with a masked last piece, and FP16 rows are held in registers up to 2048 entries and read twice
-beyond.  Conditionals of every row are compared with the FP64 oracle at the tolerance of the path."""
+(needs a GB300).  A block takes 4 to 32 rows depending on the row count, rows are read in 32-byte
+pieces with a masked last piece, and FP16 and E4M3 rows are held in registers up to 512 entries and read
+twice beyond.  Conditionals of every row are compared with the FP64 oracle at the tolerance of the path."""
 import numpy as np
 import pytest
 
@@ -23,7 +23,7 @@ def _stored(ts, precision):
 @pytest.mark.parametrize("precision", ["fp32", "bf16x2", "bf16x3l", "fp16x2"])
 @pytest.mark.parametrize("d,bonds", [
     (3, [1, 3, 1, 2, 6, 17, 33, 15, 5, 2, 1]),                # odd and one-entry blocks, next rows of 64 entries
-    (10, [1, 10, 100, 1050, 105, 11, 2, 1]),                  # a row wider than the register-resident path
+    (10, [1, 10, 100, 1050, 105, 11, 2, 1]),                  # rows of many pieces
     (255, [1, 3, 20, 1]),                                     # the most outcomes a site may have
 ])
 def test_measure_edges_against_oracle(precision, d, bonds):
@@ -116,3 +116,34 @@ def test_displacement_pairs_and_singles_give_the_same_bits(d):
             shifted = torch.empty(d * d * n + 1, dtype=torch.complex64, device="cuda")[1:]
             F.fastmps_displacement(s.h, mu[:n], d, out=shifted)
             assert np.array_equal(shifted.cpu().numpy().reshape(d, d, n), ref[:, :, :n])
+
+
+@pytest.mark.parametrize("precision", ["fp16x2", "fp16x3", "bf16x2"])
+def test_rows_around_the_piece_that_stays_in_registers(precision):
+    """Next rows of 512 entries, the widest that a warp scales without a second read, and of 576 (FP16); pieces of
+    eight entries whose last one holds 2, 4 or 6 real ones."""
+    import paper_2512_20064_gb300 as F
+
+    bonds = [1, 10, 100, 255, 256, 257, 256, 255, 97, 10, 1]
+    b, ts, _ = gen.mps_tensors(len(bonds) - 1, 10, 257, base_seed=12, skew=1.5, dtype=np.complex64, bonds=bonds)
+    stored = [quant.dequant_fp16(A, 2) for A in ts] if precision == "fp16x3" else _stored(ts, precision)
+    N = 41
+    with F.Sampler(precision=precision) as s:
+        s.load_chain(ts)
+        smp, lp, tr = s.sample(b, 10, N, 29, trace_rows=N)
+    parity.check(b, stored, 29, np.arange(N), smp, lp, 1e-4, dev_trace=tr, trace_rows=N)
+
+
+def test_small_fp32_chain_on_the_measurement_kernel():
+    """Odd and one-entry blocks of a chain that runs in one launch by itself, in micro-batches of 128 rows: the
+    stand-alone measurement kernel against the oracle."""
+    import paper_2512_20064_gb300 as F
+
+    bonds = [1, 3, 1, 2, 6, 17, 33, 15, 5, 2, 1]
+    b, ts, _ = gen.mps_tensors(len(bonds) - 1, 3, 33, base_seed=5, skew=1.5, dtype=np.complex64, bonds=bonds)
+    N = 300
+    with F.Sampler(precision="fp32", max_microbatch=128) as s:
+        s.load_chain(ts)
+        smp, lp, tr = s.sample(b, 3, N, 19, trace_rows=N)
+        assert s.stats()["contract_launches"] == 3 * len(ts)
+    parity.check(b, ts, 19, np.arange(N), smp, lp, TOL["fp32"], dev_trace=tr, trace_rows=N)
