@@ -660,7 +660,9 @@ tc_contract_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_consta
             bool failed = false;
             int mt, nt;
             for (int i = 0; !failed && tile_of<kMode, kPair>(p, i, mt, nt); ++i) {
-                const int y_a = p.row0 + mt * kBM;
+                // a pair's m-tile past the last one takes that one's rows (its own may be rows of the next micro-batch,
+                // which a measurement on the other stream may still be writing); nothing of it is stored
+                const int y_a = p.row0 + (kPair ? min(mt, p.num_m_tiles - 1) : mt) * kBM;
                 const int y_b = nt * p.bn + (int)pair_rank * (p.bn / 2);  // pair: this CTA's half of the tile's columns
                 for (int kb = kb_lo; kb < kb_hi; ++kb) {
                     if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, abort_flag)) {
