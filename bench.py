@@ -185,9 +185,9 @@ class ClockSampler:
 # DRAM bytes (read + write) of one contraction launch at an interior site, from the committed ncu
 # captures (scaled by rows to the bench's launch size); None where no capture of the current kernel exists.
 CONTRACT_TRAFFIC = {
-    ("precision", "bf16x2", "separate", 0): (2.89e9, "profiles/tc_contract_precision_bf16x2.md"),
-    ("plain", "bf16x2", "separate", 0): (1.287e9, "profiles/tc_contract_plain_bf16x2.md"),
-    ("precision", "fp16x2", "separate", 4): (2.85e9, "profiles/tc_contract_precision_fp16x2_promoted.md"),
+    ("precision", "bf16x2", "separate", 0): (3.40e9, "profiles/contract_pairs_and_others.md"),
+    ("plain", "bf16x2", "separate", 0): (1.288e9, "profiles/contract_pairs_and_others.md"),
+    ("precision", "fp16x2", "separate", 4): (3.26e9, "profiles/contract_pairs_and_others.md"),
 }
 
 

@@ -2,8 +2,9 @@
 //
 // * Vidal form (Sec. 2.2 workflow over the tensors Gamma_i; Algorithm 2 takes
 //   the coefficient vector Lambda): the site is stored as the right-canonical
-//   A_k[a, s, b] = Gamma_k[a, s, b] * Lambda_k[b], scaled in the staging copy
-//   before the repack, so that sampling runs the canonical path unchanged.
+//   A_k[a, s, b] = Gamma_k[a, s, b] * Lambda_k[b], so that sampling runs the
+//   canonical path unchanged.  FP32 and FP8 scale the staging copy before the
+//   repack (here); the 16-bit repack applies Lambda itself (kernels.cu).
 // * Displacement (Sec. 3.4.1): the displacement operator exp(mu a^+ - mu^* a)
 //   on the physical index is taken as the Zassenhaus product
 //   exp(-|mu|^2/2) exp(mu a^+) exp(-mu^* a) of a lower- and an upper-triangular
@@ -41,7 +42,7 @@
 namespace fastmps {
 
 // ---------------------------------------------------------------------------
-// Vidal form: A[a, s, b] = Gamma[a, s, b] * Lambda[b], in place on the staging copy
+// Vidal form, FP32 and FP8: A[a, s, b] = Gamma[a, s, b] * Lambda[b], in place on the staging copy
 // ---------------------------------------------------------------------------
 __global__ void scale_columns_kernel(void *A, int is_f64, int64_t n_complex, int chi_r, const void *lam) {
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n_complex;

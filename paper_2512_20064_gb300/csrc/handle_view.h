@@ -33,9 +33,9 @@ int site_view(fastmps_handle h, int k, SiteView *out);
 int set_error(fastmps_handle h, int code, const char *msg);
 // The product list of a BF16 precision mode (planes of V and B and the pairs multiplied).
 void precision_products(int precision, int *a_planes, int *b_planes, int *nprod, int *pa, int *pb);
-// cuTensorMapEncodeTiled over a BF16 matrix [outer][ld] with a (64 x box_outer) box, 128-byte swizzle.
-// FP32 scratch [rows][ld_elems] of a contraction (see encode_2d_f32_scratch).
+// Tensor map of the FP32 scratch [rows][ld_elems] of a contraction (see encode_2d_f32_scratch).
 bool encode_scratch_map(CUtensorMap *map, const void *base, uint64_t cols, uint64_t rows, uint64_t ld_elems);
+// cuTensorMapEncodeTiled over a BF16 matrix [outer][ld] with a (64 x box_outer) box, 128-byte swizzle.
 bool encode_bf16_map(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint64_t ld_elems,
                      uint32_t box_outer);
 

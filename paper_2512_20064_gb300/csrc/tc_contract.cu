@@ -22,8 +22,10 @@
 // Pair variant (kPair; two-pass and promoted): a cluster of two CTAs computes 256 rows x bn columns with
 // tcgen05 cta_group::2.  Each CTA loads its own 128 rows and half of the columns and drains its own 128 rows;
 // both CTAs' copies complete on the barriers of CTA 0, whose MMA thread issues the M = 256 products and commits
-// to both.  A CTA takes in 48 KB per k-block instead of 64 (two left planes, one site plane, bn = 256), near the
-// most an SM can (64 bytes a cycle), and holds one more pipeline stage.
+// to both.  A CTA takes in 48 KB per k-block instead of 64 (two left planes, one site plane, bn = 256: 48 bytes a
+// cycle of its products in place of 64, about what an SM can take in), and holds one more pipeline stage.  Measured,
+// K = 512, 131072 rows x 2048 columns: 343 us, tensor pipe 72 %, reads 34 and scratch stores 12 bytes a cycle and SM
+// (single CTAs: 354 us, 67 %).
 //
 // Fused variant (320 threads): warps 6-9 measure.  Each thread block owns
 // whole m-tiles (128 rows) and walks all their n-tiles in order; after the

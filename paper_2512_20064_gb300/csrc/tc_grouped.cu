@@ -2,8 +2,8 @@
 // every site, in one launch.
 //
 // The kernel is the tcgen05 contraction of tc_contract.cu (TMA producer warp,
-// MMA warp, four epilogue warps, two TMEM accumulators) with four measurement
-// warps, run over one task list: the tiles of every (job, chunk, site)
+// MMA warp, four epilogue warps, two TMEM accumulators) with eight measurement
+// warps in two groups, run over one task list: the tiles of every (job, chunk, site)
 // segment in round order.  Each task looks up its segment (tensor maps in
 // device memory, n-tile width, K extent, scratch pointers), so jobs with
 // different bond dimensions, physical dimensions and row counts share the GPU
